@@ -124,8 +124,10 @@ typedef struct lbf_dims {
   int32_t n_stokes;           /* nS: 1 (I), 4 (IQUV), 0 (voltages) */
   int32_t d_max;              /* largest integer shift d_s, in samples */
   int32_t history_samples;    /* H = (L-1) N + d_max samples kept per (station, subband) */
-  int32_t bf_kernel;          /* beam former the plan uses: 1 few-beam, 2 many-beam FP32 (128-beam
-                                 tiles), 3 tensor core, 4 many-beam FP32 (64-beam tiles) */
+  int32_t bf_kernel;          /* beam-former form of the plan: 1 few-beam, 2 many-beam FP32 (128-beam
+                                 tiles), 3 tensor core, 4 many-beam FP32 (64-beam tiles); up to 64
+                                 stations the FP32 forms of more than a few beams run on the tensor
+                                 cores from error-free FP16 slices, to FP32 accuracy */
   size_t in_bytes;            /* bytes of one input block */
   size_t chan_bytes;          /* bytes of a chan buffer */
   size_t ct_bytes;            /* bytes of a ct buffer */

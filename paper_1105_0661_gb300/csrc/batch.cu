@@ -84,6 +84,17 @@ void free_graphs(lbf_batch_t b) {
   }
 }
 
+// Whether plan i's beam former runs as the split tensor-core kernel (as it does alone).
+bool split_plan(const lbf_batch_s *b, int i) {
+  const lbf_plan_t p = b->plans[i];
+  return !p->tc && lbf::beamform_uses_split(p->geometry(), b->variant[i], p->out_kind);
+}
+
+// launch class of a tensor-core or split plan: output kind and integration length
+long long tc_class(const lbf_plan_s *p) {
+  return (long long)p->out_kind * 64 + (p->out_kind == lbf::OUT_VOLTAGES ? 1 : p->Q);
+}
+
 // Fill the group tables of parity `par` (par = 1: every plan's history one block ahead) for the
 // given block buffers: filter-bank groups class by class (work items numbered from 0 within a
 // class; history elements numbered over the whole table), then the FP32 beam-former groups class
@@ -144,7 +155,7 @@ void fill_tables(lbf_batch_t b, int par, const void *const *d_in, void *const *d
   std::vector<size_t> smem_of(n, 0);
   for (int i = 0; i < n; ++i) {
     lbf_plan_t p = b->plans[i];
-    if (p->tc) continue;
+    if (p->tc || split_plan(b, i)) continue;
     smem_of[i] = lbf::bf_smem_bytes(b->variant[i], p->S);
     per_sm[i] = lbf::bf_group_residency(b->variant[i], p->out_kind, smem_of[i]);
   }
@@ -153,11 +164,11 @@ void fill_tables(lbf_batch_t b, int par, const void *const *d_in, void *const *d
   std::vector<bool> placed(n, false);
   for (int i = 0; i < n; ++i) {
     lbf_plan_t pi = b->plans[i];
-    if (pi->tc || placed[i]) continue;
+    if (pi->tc || placed[i] || split_plan(b, i)) continue;
     lbf_batch_s::BfClass cls{b->variant[i], pi->out_kind, per_sm[i], slot, 0, 0, 0};
     for (int j = i; j < n; ++j) {
       lbf_plan_t p = b->plans[j];
-      if (p->tc || placed[j] || b->variant[j] != cls.variant || p->out_kind != cls.out_kind ||
+      if (p->tc || placed[j] || split_plan(b, j) || b->variant[j] != cls.variant || p->out_kind != cls.out_kind ||
           per_sm[j] != cls.per_sm || cls.n == lbf::kMaxGroups)
         continue;
       placed[j] = true;
@@ -223,6 +234,25 @@ cudaError_t enqueue(lbf_batch_t b, int par, cudaStream_t st) {
       if (e == cudaSuccess)
         e = lbf::launch_bf_group(c.variant, c.out_kind, b->h_bf + par * n + c.first, c.n, c.items,
                                  b->d_counter + counter++, c.smem, st);
+    // FP32 plans whose beam former is the split kernel: one persistent launch per class of output
+    // kind and integration length, then their incoherent beams
+    std::vector<bool> taken(n, false);
+    for (int i = 0; i < n && e == cudaSuccess; ++i) {
+      if (taken[i] || b->plans[i]->M == 0 || !split_plan(b, i)) continue;
+      std::vector<lbf::SplitPlanRef> cls;
+      for (int j = i; j < n && (int)cls.size() < lbf::split_max_plans_per_launch(); ++j) {
+        lbf_plan_t p = b->plans[j];
+        if (taken[j] || p->M == 0 || !split_plan(b, j) || tc_class(p) != tc_class(b->plans[i])) continue;
+        taken[j] = true;
+        cls.push_back(lbf::SplitPlanRef{p->geometry(), p->ws, b->tc_out[j]});
+      }
+      e = lbf::launch_bf_split(cls.data(), (int)cls.size(), b->plans[i]->out_kind, b->plans[i]->Q, st);
+    }
+    for (int i = 0; i < n && e == cudaSuccess; ++i) {
+      lbf_plan_t p = b->plans[i];
+      if (p->inc && p->M && split_plan(b, i))
+        e = lbf::launch_incoherent(p->geometry(), p->out_kind, p->ws, static_cast<float *>(b->tc_out[i]), st);
+    }
   }
   // tensor-core plans: their incoherent beams, then ONE persistent tcgen05 launch per class of
   // output kind and integration length (up to tc_max_plans_per_launch() plans each), whose CTAs
@@ -240,8 +270,7 @@ cudaError_t enqueue(lbf_batch_t b, int par, cudaStream_t st) {
       o.kpad = p->kpad;
       e = lbf::launch_incoherent_ct16(g, p->out_kind, o, static_cast<float *>(b->tc_out[i]), st);
     }
-    const long long cls = (long long)p->out_kind * 64 + (p->out_kind == lbf::OUT_VOLTAGES ? 1 : p->Q);
-    refs.push_back({cls, lbf::TcPlanRef{g, &p->tmap[0], &p->tmap[1], static_cast<float *>(b->tc_out[i]), p->d_err}});
+    refs.push_back({tc_class(p), lbf::TcPlanRef{g, &p->tmap[0], &p->tmap[1], static_cast<float *>(b->tc_out[i]), p->d_err}});
   }
   std::vector<bool> done(refs.size(), false);
   // per-plan mode: each tensor-core plan in its own launch (the single-plan kernel, with the plan
@@ -385,19 +414,24 @@ lbf_status lbf_batch_launches(lbf_batch_t b, int32_t *n_launches) {
   // classes of the tables last filled (lbf_batch_run, lbf_batch_capture or lbf_batch_tune)
   if (b->per_plan) {   // per plan: filter bank, history and beam former (+ incoherent beam) each
     int k = 0;
-    for (lbf_plan_t p : b->plans) k += p->M ? 3 + (p->tc && p->inc ? 1 : 0) : 0;
+    for (size_t i = 0; i < b->plans.size(); ++i) {
+      lbf_plan_t p = b->plans[i];
+      k += p->M ? 3 + (p->inc && (p->tc || split_plan(b, (int)i)) ? 1 : 0) : 0;
+    }
     *n_launches = k;
     return LBF_OK;
   }
   int tc_classes = 0;
-  std::vector<long long> seen;
-  for (lbf_plan_t p : b->plans) {
-    if (!p->tc || p->M == 0) continue;
-    const long long cls = (long long)p->out_kind * 64 + (p->out_kind == lbf::OUT_VOLTAGES ? 1 : p->Q);
+  std::vector<long long> seen[2];   // classes of the tensor-core and of the split plans
+  for (size_t i = 0; i < b->plans.size(); ++i) {
+    lbf_plan_t p = b->plans[i];
+    const bool split = split_plan(b, (int)i);
+    if ((!p->tc && !split) || p->M == 0) continue;
     int same = 0;
-    for (long long c : seen) same += c == cls;
-    if (same % lbf::tc_max_plans_per_launch() == 0) ++tc_classes;
-    seen.push_back(cls);
+    for (long long c : seen[split]) same += c == tc_class(p);
+    const int cap = split ? lbf::split_max_plans_per_launch() : lbf::tc_max_plans_per_launch();
+    if (same % cap == 0) ++tc_classes;
+    seen[split].push_back(tc_class(p));
     if (p->inc) ++tc_classes;   // its incoherent-beam kernel
   }
   *n_launches = (int32_t)(b->ppf_cls.size() + 1 + b->bf_cls.size()) + tc_classes;

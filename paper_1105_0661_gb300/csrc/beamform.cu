@@ -5,7 +5,8 @@
 // with w[b,s] = exp(+2 pi i f_c dtau[b,s]), f_c = f0_f + df_c.  The weights are generated per CTA
 // into shared memory from the plan's FP64-reduced phase tables (tables.cu) and an FP32 sincos.
 //
-// Two kernels:
+// Up to 64 stations most of this runs as the split tensor-core kernel (bf_split.cu,
+// beamform_uses_split); the FP32 FMA kernels here serve few beams and more stations:
 //  * few-beam (bandwidth bound): one thread per spectrum m (both pols), weights broadcast from
 //    shared memory, one coalesced pass over the corner-turned input; Stokes integration over Q
 //    consecutive spectra is a warp-shuffle reduction across the lanes that hold them.
@@ -421,11 +422,62 @@ cudaError_t launch_many(const Geometry &g, int out_kind, const float2 *ct, void 
   }
 }
 
+// Incoherent beam from the corner-turned block, beside the split kernel: one thread per spectrum,
+// one pass over the block.
+template <int NS>
+__global__ void __launch_bounds__(kFewThreads)
+incoherent_kernel(Geometry g, const float2 *__restrict__ ct, float *__restrict__ out) {
+  const int fc = blockIdx.x, f = fc / kN, c = fc - f * kN;
+  const float2 *y = ct + (long long)fc * g.S * kP * g.M;
+  const int Mq = g.M / g.Q;
+  for (int mb = 0; mb < g.M; mb += kFewThreads) {
+    const int m = mb + threadIdx.x;
+    const bool active = m < g.M;
+    IncAcc ia;
+    if (active) {
+#pragma unroll 8
+      for (int s = 0; s < g.S; ++s) ia.add(y[((long long)s * kP) * g.M + m], y[((long long)s * kP + 1) * g.M + m]);
+    }
+#pragma unroll
+    for (int st = 0; st < NS; ++st) {
+      float v = ia.param(st);
+      for (int o2 = 1; o2 < g.Q; o2 <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o2);
+      if (active && (m & (g.Q - 1)) == 0)
+        out[((((long long)g.B * NS + st) * g.F + f) * kN + c) * Mq + m / g.Q] = v;
+    }
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct, float *out, cudaStream_t st) {
+  if ((long long)g.F * kN == 0 || g.M == 0) return cudaSuccess;
+  if (out_kind == OUT_STOKES_IQUV) incoherent_kernel<4><<<g.F * kN, kFewThreads, 0, st>>>(g, ct, out);
+  else incoherent_kernel<1><<<g.F * kN, kFewThreads, 0, st>>>(g, ct, out);
+  return cudaGetLastError();
+}
+
+// The split kernel takes the many-beam forms up to 64 stations, and of the few-beam form (Stokes
+// outputs) what would be two passes or more of the few-beam kernel over enough stations: its time
+// hardly depends on the beams up to 64, the few-beam kernel's grows with passes x stations.  Measured
+// for 16 subbands of 768 spectra, Stokes I, few-beam / split: 8 stations 16 beams 0.33 / 0.40 ms and
+// 32 beams 0.66 / 0.40; 16 stations 16 beams 0.47 / 0.42; 48 stations 8 beams 0.52 / 0.59 and 16
+// beams 0.99 / 0.59; voltages of 48 stations, 16 beams (8 subbands) 0.60 / 0.94.
+bool beamform_uses_split(const Geometry &g, int variant, int out_kind) {
+  if (g.S > split_max_stations()) return false;
+  if (variant != 1) return true;
+  return out_kind != OUT_VOLTAGES && g.B > 8 && (g.B + 7) / 8 * g.S >= 24;
+}
 
 cudaError_t launch_beamform(const Geometry &g, int variant, int out_kind, const float2 *ct, void *out,
                             cudaStream_t st) {
   if ((long long)g.F * kN == 0 || g.M == 0 || g.B == 0) return cudaSuccess;
+  if (beamform_uses_split(g, variant, out_kind)) {
+    const SplitPlanRef r{g, ct, out};
+    const cudaError_t e = launch_bf_split(&r, 1, out_kind, g.Q, st);
+    if (e != cudaSuccess || !g.inc || out_kind == OUT_VOLTAGES) return e;
+    return launch_incoherent(g, out_kind, ct, static_cast<float *>(out), st);
+  }
   // Stokes I: 16 beams per CTA where that makes fewer passes per cost -- a 16-beam CTA costs ~1.91
   // of an 8-beam one (measured on the LOFAR block: the same reads, twice the arithmetic), so 9-16
   // and 25-32 beams gain 4-9 % and 17-24 would lose.  Voltages and IQUV keep 8 (their 16-beam

@@ -71,6 +71,21 @@ cudaError_t encode_ct32_store_map(void *map, void *base, int S, int M, long long
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+cudaError_t encode_ct32_tile_map(void *map, const void *base, int rows, int M, long long fc_rows, int nsp) {
+  PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+  if (!encode) return cudaErrorNotSupported;
+  if (M % 2 != 0 || rows < 1 || rows > 256 || nsp < 2 || nsp > 128) return cudaErrorInvalidValue;
+  const cuuint64_t row = (cuuint64_t)M * 8;
+  const cuuint64_t dims[3] = {(cuuint64_t)M * 2, (cuuint64_t)rows, (cuuint64_t)fc_rows};
+  const cuuint64_t strides[2] = {row, row * (cuuint64_t)rows};
+  const cuuint32_t box[3] = {2 * (cuuint32_t)nsp, (cuuint32_t)rows, 1};
+  const cuuint32_t elem[3] = {1, 1, 1};
+  CUresult r = encode(static_cast<CUtensorMap *>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(base), dims,
+                      strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 }  // namespace lbf
 
 namespace {
@@ -372,7 +387,7 @@ lbf_status lbf_plan(const lbf_config *cfg, lbf_plan_t *out) {
   if (e == cudaSuccess) e = upload(&p->resid, resid.data(), resid.size());
   if (e == cudaSuccess) e = upload(&p->f0, cfg->subband_centre_hz, (size_t)p->F);
   if (e == cudaSuccess) e = upload(&p->dtau, dtau.data(), dtau.size());
-  if (e == cudaSuccess) e = upload<float>(&p->phase0, nullptr, (size_t)p->F * p->B * p->S);
+  if (e == cudaSuccess) e = upload<int>(&p->phase0, nullptr, (size_t)p->F * p->B * p->S);
   if (e == cudaSuccess) e = upload<float>(&p->step, nullptr, (size_t)p->B * p->S);
   if (e == cudaSuccess) e = lbf::launch_phase_tables(p->F, p->B, p->S, p->fs, p->f0, p->dtau, p->phase0, p->step, 0);
   p->hist_bytes = (size_t)p->S * p->F * p->H * p->word;
@@ -383,7 +398,7 @@ lbf_status lbf_plan(const lbf_config *cfg, lbf_plan_t *out) {
   p->tc = tc_asked && !tc_few;
   p->tc_wlo = cfg->precision == LBF_FP16_TC2 ? 0 : 1;
   if (p->tc) {   // weight tables with the delay compensation folded in, for the fused path
-    if (e == cudaSuccess) e = upload<float>(&p->phase0g, nullptr, (size_t)p->F * p->B * p->S);
+    if (e == cudaSuccess) e = upload<int>(&p->phase0g, nullptr, (size_t)p->F * p->B * p->S);
     if (e == cudaSuccess) e = upload<float>(&p->stepg, nullptr, (size_t)p->B * p->S);
     if (e == cudaSuccess)
       e = lbf::launch_phase_tables(p->F, p->B, p->S, p->fs, p->f0, p->dtau, p->phase0g, p->stepg, 0, p->tau,

@@ -27,11 +27,11 @@ struct Geometry {
   const double *resid = nullptr;        // [S] tau_s - n_s Ts
   const double *f0 = nullptr;           // [F] subband centre frequency
   const double *dtau = nullptr;         // [B][S] beam delay difference
-  const float *phase0 = nullptr;        // [F][B][S] f0_f dtau[b,s] reduced to [-1/2, 1/2] cycle (FP64 -> FP32)
+  const int *phase0 = nullptr;          // [F][B][S] f0_f dtau[b,s] modulo one cycle, in 2^-32 cycle (from FP64)
   const float *step = nullptr;          // [B][S] fs/N * dtau[b,s], cycles per channel
   // the same two tables with the delay compensation folded in (tensor-core plans): phase
   // f0_f (dtau[b,s] + tau_s) reduced, step fs/N (dtau[b,s] + tau_s - n_s Ts)
-  const float *phase0g = nullptr;
+  const int *phase0g = nullptr;
   const float *stepg = nullptr;
   int ct16_raw = 0;           // 1: the FP16 planes hold the filtered spectrum before the delay phase
                               // and bandpass, which the tensor-core weights then carry
@@ -61,6 +61,9 @@ cudaError_t encode_ct16_store_map(void *map, void *base, int kpad, int M, long l
 // The same for the FP32 corner turn [F*N][S][P][M] float2 (M even): boxes of 16 spectra of one
 // (station, pol) x `nch` consecutive channels.
 cudaError_t encode_ct32_store_map(void *map, void *base, int S, int M, long long fc_rows, int nch);
+// ... and as [F*N][rows = S*P][M] float2 for the split beam former's prefetches: boxes of `nsp`
+// spectra of all rows of one channel.
+cudaError_t encode_ct32_tile_map(void *map, const void *base, int rows, int M, long long fc_rows, int nsp);
 
 // One observation of a batch (grouped persistent launches, batch.cu): its geometry, this
 // block's buffers, and its range of work items in the grouped filter bank and beam former.
@@ -175,9 +178,24 @@ cudaError_t launch_delay_ct(const Geometry &g, const float2 *chan, float2 *ct, c
 // (128-beam tiles), 3 many (64-beam tiles)
 cudaError_t launch_beamform(const Geometry &g, int variant, int out_kind, const float2 *ct,
                             void *out, cudaStream_t st);
+// FP32 beam former on the tensor cores by an error-free split (bf_split.cu), for up to
+// split_max_plans_per_launch() plans of one output kind and integration length in one persistent
+// launch; the incoherent beam of a plan that has one is not included
+struct SplitPlanRef {
+  Geometry g;
+  const float2 *ct;
+  void *out;
+};
+cudaError_t launch_bf_split(const SplitPlanRef *plans, int n, int out_kind, int Q, cudaStream_t st);
+int split_max_stations();
+int split_max_plans_per_launch();
+// whether launch_beamform runs `variant` of this observation as the split kernel
+bool beamform_uses_split(const Geometry &g, int variant, int out_kind);
+// incoherent beam (index B of the Stokes output) from the FP32 corner-turned block
+cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct, float *out, cudaStream_t st);
 // plan-time FP64 tables of the weight phases (tables.cu)
 cudaError_t launch_phase_tables(int F, int B, int S, double fs, const double *f0, const double *dtau,
-                                float *phase0, float *step, cudaStream_t st, const double *tau = nullptr,
+                                int *phase0, float *step, cudaStream_t st, const double *tau = nullptr,
                                 const double *resid = nullptr);
 // largest S the many-beam kernel accepts (shared-memory bound)
 int many_beam_max_stations();
@@ -199,13 +217,27 @@ __device__ __forceinline__ float2 unit_phasor_cycles(double phi) {
   return make_float2(c, s);
 }
 
-// Weight w[b,s] of channel c (Section 4.3) from the plan's phase tables: the FP64-reduced carrier
-// phase of (f, b, s) plus the FP32 channel term, through an FP32 sincos.
+// Phase of a weight in 2^-32 cycle: the table's carrier phase plus dc channels of `step` cycles.
+__device__ __forceinline__ int weight_phase(int phase0, float step, float dc) {
+  float x = dc * step;
+  x -= rintf(x);
+  return (int)((unsigned)phase0 + (unsigned)__float2int_rn(x * 4294967296.0f));
+}
+
+// exp(2 pi i phi) of a phase in 2^-32 cycle: reduced to the nearest quarter cycle in integers, so
+// the FP32 argument is at most 1/8 cycle (an eighth of a cycle in FP32 is good to 4e-9 cycle).
+__device__ __forceinline__ float2 fixed_phasor(int phi) {
+  const int q = (int)((unsigned)phi + (1u << 29)) >> 30;
+  const int r = (int)((unsigned)phi - ((unsigned)q << 30));
+  float s, c;
+  sincospif((float)r * 4.656612873077393e-10f, &s, &c);   // 2 x 2^-32 half turns
+  const float x = (q & 1) ? -s : c, y = (q & 1) ? c : s;
+  return (q & 2) ? make_float2(-x, -y) : make_float2(x, y);
+}
+
+// Weight w[b,s] of channel c (Section 4.3) from the plan's phase tables.
 __device__ __forceinline__ float2 beam_weight(const Geometry &g, int f, int c, long long bs) {
-  const float phi = fmaf((float)(c - kN / 2), g.step[bs], g.phase0[(long long)f * g.B * g.S + bs]);
-  float s, co;
-  sincospif(2.0f * phi, &s, &co);
-  return make_float2(co, s);
+  return fixed_phasor(weight_phase(g.phase0[(long long)f * g.B * g.S + bs], g.step[bs], (float)(c - kN / 2)));
 }
 
 }  // namespace lbf

@@ -24,8 +24,9 @@ struct lbf_plan_s {
   float *bandpass = nullptr;
   int *dshift = nullptr;
   double *tau = nullptr, *resid = nullptr, *f0 = nullptr, *dtau = nullptr;
-  float *phase0 = nullptr, *step = nullptr;
-  float *phase0g = nullptr, *stepg = nullptr;   // with the delay folded in (tensor-core plans)
+  int *phase0 = nullptr, *phase0g = nullptr;
+  float *step = nullptr;
+  float *stepg = nullptr;   // with the delay folded in (tensor-core plans)
   // tensor-core precision: FP16 corner-turned planes and their TMA descriptors
   bool tc = false;
   int tc_wlo = 1;               // three products (LBF_FP16_TC) or two (LBF_FP16_TC2)

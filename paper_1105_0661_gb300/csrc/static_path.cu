@@ -180,13 +180,13 @@ extern "C" lbf_status lbf_run_block_static(const lbf_config *c, const void *d_in
   g.resid = reinterpret_cast<const double *>(tab + tm.resid);
   g.f0 = reinterpret_cast<const double *>(tab + tm.f0);
   g.dtau = reinterpret_cast<const double *>(tab + tm.dtau);
-  g.phase0 = reinterpret_cast<const float *>(tab + tm.phase0);
+  g.phase0 = reinterpret_cast<const int *>(tab + tm.phase0);
   g.step = reinterpret_cast<const float *>(tab + tm.step);
   g.err = reinterpret_cast<int *>(tab + tm.err);
   const int out_kind = c->output == LBF_STOKES_I ? lbf::OUT_STOKES_I
                      : c->output == LBF_STOKES_IQUV ? lbf::OUT_STOKES_IQUV : lbf::OUT_VOLTAGES;
   if (e == cudaSuccess)
-    e = lbf::launch_phase_tables(F, B, S, g.fs, g.f0, g.dtau, reinterpret_cast<float *>(tab + tm.phase0),
+    e = lbf::launch_phase_tables(F, B, S, g.fs, g.f0, g.dtau, reinterpret_cast<int *>(tab + tm.phase0),
                                  reinterpret_cast<float *>(tab + tm.step), st);
   if (e == cudaSuccess) e = lbf::launch_ppf(g, c->sample_bits, d_in, hist, nullptr, ct, st);
   if (e == cudaSuccess) e = lbf::launch_beamform(g, variant, out_kind, ct, d_out, st);
