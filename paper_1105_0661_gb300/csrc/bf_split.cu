@@ -245,43 +245,12 @@ __device__ __forceinline__ void flush_stage(const SpParams &p, const float *buf,
   }
 }
 
-// Short windows (Q < 8) go through the warp's own 4 KB: rows of up to 16 windows, a row per beam (I)
-// or per lane (IQUV: ro 0 holds I and Q, ro 1 U and V, in two buffers), the window index XORed so
-// that neither walk meets a bank twice, then to global memory a run of windows per row.
-template <int NS, int Q>
-struct ShortRows {
-  static constexpr int kFlushCh = Q == 1 ? 1 : 2;                // 16-spectrum chunks per flush
-  static constexpr int kW = 16 * kFlushCh / Q;                   // windows per flush: 16, 16, 8
-  __device__ static int index(int row, int w) {                  // NS 4: row = lane; NS 1: row = beam
-    if (NS == 1) return row * kW + (w ^ ((2 * (row / (32 / kW))) & (kW - 1)));
-    return row * kW + (w ^ ((row / (32 / kW)) & (kW - 1)));
-  }
+// Windows per flush of the short rows: one or both 16-spectrum chunks of a half tile (16, 16, 8).
+template <int Q>
+struct Short {
+  static constexpr int kFlushCh = Q == 1 ? 1 : 2;
+  static constexpr int kW = 16 * kFlushCh / Q;
 };
-
-template <int NS, int Q>
-__device__ __forceinline__ void flush_rows(const float *stage, int lane, int nbeams, int w0, int Mq, float *row0,
-                                           long long bstride, long long pstride) {
-  using R = ShortRows<NS, Q>;
-  constexpr int kRowsPer = 32 / R::kW;                            // rows per store instruction
-  const int w = lane % R::kW, rl = lane / R::kW;
-  __syncwarp();
-#pragma unroll
-  for (int k = 0; k < (NS == 1 ? 16 : 32) / kRowsPer; ++k) {
-    const int row = k * kRowsPer + rl;
-    const int jq = NS == 1 ? row : row >> 1;
-    if (jq < nbeams && w0 + w < Mq) {
-      float *dst = row0 + (long long)jq * bstride + w0 + w;
-      if (NS == 1) {
-        dst[0] = stage[R::index(row, w)];
-      } else {
-        dst += (row & 1) * 2 * pstride;
-        dst[0] = stage[R::index(row, w)];
-        dst[pstride] = stage[512 + R::index(row, w)];
-      }
-    }
-  }
-  __syncwarp();   // the rows are rewritten by the next chunk
-}
 
 // Stokes parameters of one 32-spectrum half tile (spectra m0 .. m0 + 31) from this lane's voltage
 // component (Re rows ro = 0, Im rows ro = 1): vx, vy hold pairs of spectra of pol X and Y.  Windows of
@@ -323,14 +292,7 @@ __device__ __forceinline__ void stokes_half(const float2 (&vx)[16], const float2
           }
         }
       } else {
-        using R = ShortRows<NS, Q>;
-        const int wf = R::kFlushCh == 2 ? ch * kW + w : w;
-        if (NS == 1) {
-          if ((wf & 1) == ro) wstage[R::index(jq, wf)] = r0;
-        } else {
-          wstage[R::index(lane, wf)] = r0;
-          wstage[512 + R::index(lane, wf)] = r1;
-        }
+        ShortRows<NS, Short<Q>::kW>::put(wstage, lane, Short<Q>::kFlushCh == 2 ? ch * kW + w : w, r0, r1);
       }
     };
 #pragma unroll
@@ -355,8 +317,9 @@ __device__ __forceinline__ void stokes_half(const float2 (&vx)[16], const float2
       }
     }
     if constexpr (!Stage<NS, Q>::kOn)
-      if (ShortRows<NS, Q>::kFlushCh == 1 || ch == 1)
-        flush_rows<NS, Q>(wstage, lane, nbeams, ShortRows<NS, Q>::kFlushCh == 1 ? w0 : m0 / Q, Mq, row0, bstride, pstride);
+      if (Short<Q>::kFlushCh == 1 || ch == 1)
+        ShortRows<NS, Short<Q>::kW>::flush(wstage, lane, nbeams, Short<Q>::kFlushCh == 1 ? w0 : m0 / Q, Mq, row0, bstride,
+                                           pstride);
   }
 }
 

@@ -70,8 +70,7 @@ struct TcParams {
   int stage_bytes;            // its ring stage: 2 planes x 2 tiles x Kpad K rows x 128 bytes
   int vec;                    // output rows 16-byte aligned (M/Q % 4 == 0, aligned base)
   int wlo;                    // 1: three products (Wlo Yhi too); 0: two products
-  const int *phase0;
-  const float *step;
+  const float *phase0, *step;
   const float *bp;            // bandpass applied to the outputs (raw FP16 planes), or null
   float *out;
   int *err;                   // the plan's device error word
@@ -119,7 +118,7 @@ __device__ __forceinline__ void load_weight_tables(const TcParams &p, int f, int
     const int s = (half + KS * (i >> 2)) * 8 + 2 * (i & 3) + ro;
     const bool ok = b < p.B && s < p.S;
     const long long bs = (long long)b * p.S + s;
-    w.ph[i] = ok ? (float)__ldg(&p.phase0[(long long)f * p.B * p.S + bs]) * 2.3283064365386963e-10f : 0.f;
+    w.ph[i] = ok ? __ldg(&p.phase0[(long long)f * p.B * p.S + bs]) : 0.f;
     w.st[i] = ok ? __ldg(&p.step[bs]) : 0.f;
     w.ok |= (ok ? 1u : 0u) << i;
   }
@@ -167,33 +166,40 @@ __device__ __forceinline__ void write_weights(const TcParams &p, uint32_t ta_hi,
 
 constexpr int kVStageBytes = 8 * 2 * kSpec * 8;   // voltages: 8 beams x 2 pols x 32 spectra, cf32
 
-// Output staging.  For Q >= 8 the epilogue collects 8 consecutive windows of every (beam, Stokes
-// parameter) row of its lane quadrant in shared memory and then writes each row segment as two
-// 16-byte stores (a whole 32-byte sector), instead of scattering 4-byte stores over rows that lie
-// megabytes apart.  A quadrant's buffer: 32 beams (16 per M tile) x NS parameters x 8 windows,
-// the 16-byte chunks of a beam XOR-swizzled by the beam index; two buffers alternate.
+// Output staging.  For Q >= 4 the epilogue collects 8 (16 for Q = 4, a whole tile pair) consecutive
+// windows of every (beam, Stokes parameter) row of its lane quadrant in shared memory and then writes
+// each row segment as 16-byte stores (whole 32-byte sectors), instead of scattering 4-byte stores
+// over rows that lie megabytes apart.  A quadrant's buffer: 32 beams (16 per M tile) x NS parameters x
+// kWin windows, the 16-byte chunks of a beam XOR-swizzled by the beam index; two buffers alternate.
+// Shorter windows go through each warp's short rows (tc_ptx.cuh).  Measured, 300 beams IQUV over 4 of
+// 40 stations, 24 subbands of 384 spectra (2.8 GB of output): 9.73 ms with the
+// scattered stores, 1.94 staged; 128 beams IQUV unintegrated: 32.1 and 1.87.
 template <int NS, int Q>
 struct Stage {
-  static constexpr bool kOn = Q >= 8;
+  static constexpr bool kOn = NS != 0 && Q >= 4;
   static constexpr int kPeriod = Q >= 8 ? Q / 8 : 1;          // tile pairs per flush
-  static constexpr int kRow = NS * 8;                          // floats per beam (0: voltages)
+  static constexpr int kWin = Q >= 8 ? 8 : 16;                 // windows per flush
+  static constexpr int kParts = kWin / 4;                      // 16-byte parts of a row segment
+  static constexpr int kRow = NS * kWin;                       // floats per beam (0: voltages)
   static constexpr int kBuf = 32 * kRow;                       // floats per quadrant buffer
+  using Rows = ShortRows<NS == 0 ? 1 : NS, Q <= 2 ? 16 / Q : 8>;
   static constexpr int kBytes = NS == 0 ? 8 * kVStageBytes       // voltages: 4 KB per epilogue warp
-                                        : kOn ? 4 * 2 * kBuf * 4 : 0;   // 4 quadrants x 2 buffers
+                                        : kOn ? 4 * 2 * kBuf * 4   // 4 quadrants x 2 buffers
+                                              : 4 * epi_split<NS, Q>() * Rows::kBytes;
   __device__ static int index(int jq, int param, int wl) {     // float index within a beam's row
-    const int chunk = (param * 2 + (wl >> 2)) ^ (jq & (2 * NS - 1));
+    const int chunk = (param * kParts + (wl >> 2)) ^ (jq & (NS * kParts - 1));
     return chunk * 4 + (wl & 3);
   }
 };
 
 // kSpecW spectra (32 or 16) of one 32-spectrum tile of an accumulator (pol X at `taddr`, pol Y
 // 32 columns on; spectra m0 .. m0 + kSpecW - 1): integrate over windows of Q <= kSpecW spectra and
-// store the Stokes parameters, to the staging row `srow` (window wl = w - wbase) or, when staging
-// is off, to the output rows at `orow`; every parameter is scaled by `osc` (the squared bandpass
+// store the Stokes parameters, to the staging row `srow` (window wl = w - wbase) or, for Q < 4, to
+// the warp's short rows at `srow`; every parameter is scaled by `osc` (the squared bandpass
 // of the channel when the weights leave it out).
 template <int NS, int Q, int kSpecW>
-__device__ __forceinline__ void drain_tile(uint32_t taddr, int m0, int ro, int jq, int M, bool beam_ok, float *orow,
-                                           long long pstride, float *srow, int wbase, float osc) {
+__device__ __forceinline__ void drain_tile(uint32_t taddr, int m0, int ro, int jq, int M, bool beam_ok, float *srow,
+                                           int wbase, float osc) {
   float x[kSpecW / 16][16], y[kSpecW / 16][16];
 #pragma unroll
   for (int ch = 0; ch < kSpecW / 16; ++ch) {
@@ -209,10 +215,8 @@ __device__ __forceinline__ void drain_tile(uint32_t taddr, int m0, int ro, int j
     if (NS == 1) {
       const float i_own = sxx + syy;
       const float I = osc * (i_own + __shfl_xor_sync(0xffffffffu, i_own, 1));
-      if (ok && ro == 0) {
-        if (Stage<NS, Q>::kOn) srow[Stage<NS, Q>::index(jq, 0, w - wbase)] = I;
-        else orow[w] = I;
-      }
+      if constexpr (!Stage<NS, Q>::kOn) Stage<NS, Q>::Rows::put(srow, 2 * jq + ro, ml / Q, I, 0.f);
+      else if (ok && ro == 0) srow[Stage<NS, Q>::index(jq, 0, w - wbase)] = I;
     } else {
       // lane ro 0 ends with (I, Q), lane ro 1 with (U, V): each sends what its partner keeps
       const float i_own = sxx + syy, q_own = sxx - syy, u_own = sxy, v_own = ro ? sv : -sv;
@@ -223,15 +227,12 @@ __device__ __forceinline__ void drain_tile(uint32_t taddr, int m0, int ro, int j
       const float sc = ro ? 2.f * osc : osc;
       k0 *= sc;
       k1 *= sc;
-      if (ok) {
+      if constexpr (!Stage<NS, Q>::kOn) {
+        Stage<NS, Q>::Rows::put(srow, 2 * jq + ro, ml / Q, k0, k1);
+      } else if (ok) {
         const int p0 = ro ? 2 : 0;
-        if (Stage<NS, Q>::kOn) {
-          srow[Stage<NS, Q>::index(jq, p0, w - wbase)] = k0;
-          srow[Stage<NS, Q>::index(jq, p0 + 1, w - wbase)] = k1;
-        } else {
-          orow[p0 * pstride + w] = k0;
-          orow[(p0 + 1) * pstride + w] = k1;
-        }
+        srow[Stage<NS, Q>::index(jq, p0, w - wbase)] = k0;
+        srow[Stage<NS, Q>::index(jq, p0 + 1, w - wbase)] = k1;
       }
     }
   };
@@ -336,12 +337,13 @@ __device__ __forceinline__ void drain_tile_v(uint32_t taddr, int m0, int ro, int
 
 // The rows a thread writes in every flush of a work item (kQT threads per quadrant: thread tq of
 // the quadrant's epilogue warps): rows (beam, Stokes parameter) i = tq + kQT k, each written as the
-// 16-byte part `part` of a 32-byte segment.  Their addresses depend only on the item, so they are
-// formed once per item (null for beams past B, and for threads past the quadrant's 64 NS parts).
+// 16-byte part `part` of a segment.  Their addresses depend only on the item, so they are
+// formed once per item (null for beams past B, and for threads past the quadrant's 32 NS kParts parts).
 template <int NS, int Q>
 struct FlushRows {
   static constexpr int kQT = 32 * epi_split<NS, Q>();
-  static constexpr int kRowsPer = NS * 2 * 32 / kQT > 0 ? NS * 2 * 32 / kQT : 1;   // rows per thread
+  static constexpr int kAll = NS * Stage<NS, Q>::kParts * 32;
+  static constexpr int kRowsPer = kAll / kQT > 0 ? kAll / kQT : 1;   // rows per thread
   float *row[kRowsPer];
   int soff[kRowsPer];     // float offset of the row's part within the quadrant buffer
   int part;
@@ -351,20 +353,21 @@ template <int NS, int Q>
 __device__ __forceinline__ void flush_rows(const TcParams &p, FlushRows<NS, Q> &fr, int tq, int quad, int bb, int f,
                                            int c) {
   const int Mq = p.M / Q;
-  fr.part = tq & 1;
+  constexpr int kParts = Stage<NS, Q>::kParts;
+  fr.part = tq % kParts;
 #pragma unroll
   for (int k = 0; k < FlushRows<NS, Q>::kRowsPer; ++k) {
     const int i = tq + FlushRows<NS, Q>::kQT * k;
-    const int param = (i >> 1) % NS, bq = (i >> 1) / NS;
+    const int param = (i / kParts) % NS, bq = (i / kParts) / NS;
     const int jq = bq & 15, mt = bq >> 4;
     const int b = bb * kBeamsPerItem + mt * (kRows / 2) + quad * 16 + jq;
-    fr.row[k] = (i < 32 * NS * 2 && b < p.B) ? p.out + ((((long long)b * NS + param) * p.F + f) * kN + c) * Mq
+    fr.row[k] = (i < FlushRows<NS, Q>::kAll && b < p.B) ? p.out + ((((long long)b * NS + param) * p.F + f) * kN + c) * Mq
                                               : nullptr;
-    fr.soff[k] = bq * Stage<NS, Q>::kRow + ((param * 2 + fr.part) ^ (jq & (2 * NS - 1))) * 4;
+    fr.soff[k] = bq * Stage<NS, Q>::kRow + ((param * kParts + fr.part) ^ (jq & (NS * kParts - 1))) * 4;
   }
 }
 
-// Write a quadrant's staged windows wbase .. wbase + 7 to the output rows.
+// Write a quadrant's staged windows wbase .. wbase + kWin - 1 to the output rows.
 template <int NS, int Q>
 __device__ __forceinline__ void flush_stage(const TcParams &p, const float *buf, const FlushRows<NS, Q> &fr,
                                             int wbase) {
@@ -583,7 +586,7 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
       FlushRows<NS, Q> frows;
       if constexpr (St::kOn) flush_rows<NS, Q>(p, frows, half * 32 + lane, quad, bb, f, c);   // tq
       for (int t = 0; t < p.ntiles && ok; ++t, gpar ^= 1u) {
-        const int wbase = (t / St::kPeriod) * 8;
+        const int wbase = (t / St::kPeriod) * St::kWin;
         float *const buf = qbuf + (fl & 1) * St::kBuf;
         for (int mt = 0; mt < kMTiles; ++mt) {
           // write the next item's weights after this tile pair: with one weight set, after the
@@ -605,13 +608,18 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
             drain_tile_v(taddr, m0, ro, jq, lane, p.M, p.B, b0, v0, bstride, p.vec != 0,
                          reinterpret_cast<float2 *>(stage_out) + (warp - 2) * (kVStageBytes / 8), bpc);
           } else {
-            float *const orow = p.out + (((long long)b * NS * p.F + f) * kN + c) * Mq;
-            drain_tile<NS, Q, kSpecW>(taddr, m0, ro, jq, p.M, b < p.B, orow, pstride, buf + (mt * 16 + jq) * St::kRow,
-                                      wbase, bpc * bpc);
+            float *const srow = St::kOn ? buf + (mt * 16 + jq) * St::kRow
+                                        : stage_out + (warp - 2) * (St::Rows::kBytes / 4);
+            drain_tile<NS, Q, kSpecW>(taddr, m0, ro, jq, p.M, b < p.B, srow, wbase, bpc * bpc);
           }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(acce_bar(mt));
+          if constexpr (NS != 0 && !St::kOn) {   // the accumulator is free: write the short rows out
+            const int b0 = bb * kBeamsPerItem + mt * (kRows / 2) + quad * 16;
+            St::Rows::flush(stage_out + (warp - 2) * (St::Rows::kBytes / 4), lane, p.B - b0, m0 / Q, Mq,
+                            p.out + (((long long)b0 * NS * p.F + f) * kN + c) * Mq, NS * pstride, pstride);
+          }
           if (boundary) {
             const uint32_t ta_hi = tmem + lane_off + wcol<kForm>(mt, (eit + 1) & 1);
             write_weights(pn, ta_hi, ta_hi + 64u, nfc % kN, ro, half, tab, wlo_of(pn));
@@ -697,7 +705,7 @@ bool fill_plan(TcLaunch &L, int i, const Geometry &g, int out_kind, const void *
   p.first_item = (int)first;
   // raw planes (the fused path): weights with the delay compensation folded in, outputs scaled by
   // the bandpass
-  p.phase0 = g.ct16_raw ? g.phase0g : g.phase0;
+  p.phase0 = g.ct16_raw ? g.phase0g : g.phase0t;
   p.step = g.ct16_raw ? g.stepg : g.step;
   p.bp = g.ct16_raw ? g.bandpass : nullptr;
   if (!p.phase0 || !p.step) return false;

@@ -124,7 +124,7 @@ void release(lbf_plan_s *p) {
   cudaFree(p->taps); cudaFree(p->twiddle); cudaFree(p->bandpass); cudaFree(p->dshift);
   cudaFree(p->tau); cudaFree(p->resid); cudaFree(p->f0); cudaFree(p->dtau);
   cudaFree(p->hist[0]); cudaFree(p->hist[1]); cudaFree(p->ws);
-  cudaFree(p->phase0); cudaFree(p->step); cudaFree(p->phase0g); cudaFree(p->stepg);
+  cudaFree(p->phase0); cudaFree(p->phase0t); cudaFree(p->step); cudaFree(p->phase0g); cudaFree(p->stepg);
   cudaFree(p->ct16[0]); cudaFree(p->d_err); cudaFree(p->ss_members); cudaFree(p->ss_offs);
   if (p->h2d) cudaStreamDestroy(p->h2d);
   if (p->d2h) cudaStreamDestroy(p->d2h);
@@ -387,9 +387,7 @@ lbf_status lbf_plan(const lbf_config *cfg, lbf_plan_t *out) {
   if (e == cudaSuccess) e = upload(&p->resid, resid.data(), resid.size());
   if (e == cudaSuccess) e = upload(&p->f0, cfg->subband_centre_hz, (size_t)p->F);
   if (e == cudaSuccess) e = upload(&p->dtau, dtau.data(), dtau.size());
-  if (e == cudaSuccess) e = upload<int>(&p->phase0, nullptr, (size_t)p->F * p->B * p->S);
   if (e == cudaSuccess) e = upload<float>(&p->step, nullptr, (size_t)p->B * p->S);
-  if (e == cudaSuccess) e = lbf::launch_phase_tables(p->F, p->B, p->S, p->fs, p->f0, p->dtau, p->phase0, p->step, 0);
   p->hist_bytes = (size_t)p->S * p->F * p->H * p->word;
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
     e = cudaMalloc(&p->hist[i], p->hist_bytes ? p->hist_bytes : 16);
@@ -397,8 +395,15 @@ lbf_status lbf_plan(const lbf_config *cfg, lbf_plan_t *out) {
   }
   p->tc = tc_asked && !tc_few;
   p->tc_wlo = cfg->precision == LBF_FP16_TC2 ? 0 : 1;
+  if (p->tc) {
+    if (e == cudaSuccess) e = upload<float>(&p->phase0t, nullptr, (size_t)p->F * p->B * p->S);
+    if (e == cudaSuccess) e = lbf::launch_phase_tables(p->F, p->B, p->S, p->fs, p->f0, p->dtau, p->phase0t, p->step, 0);
+  } else {
+    if (e == cudaSuccess) e = upload<int>(&p->phase0, nullptr, (size_t)p->F * p->B * p->S);
+    if (e == cudaSuccess) e = lbf::launch_phase_tables(p->F, p->B, p->S, p->fs, p->f0, p->dtau, p->phase0, p->step, 0);
+  }
   if (p->tc) {   // weight tables with the delay compensation folded in, for the fused path
-    if (e == cudaSuccess) e = upload<int>(&p->phase0g, nullptr, (size_t)p->F * p->B * p->S);
+    if (e == cudaSuccess) e = upload<float>(&p->phase0g, nullptr, (size_t)p->F * p->B * p->S);
     if (e == cudaSuccess) e = upload<float>(&p->stepg, nullptr, (size_t)p->B * p->S);
     if (e == cudaSuccess)
       e = lbf::launch_phase_tables(p->F, p->B, p->S, p->fs, p->f0, p->dtau, p->phase0g, p->stepg, 0, p->tau,

@@ -29,9 +29,11 @@ struct Geometry {
   const double *dtau = nullptr;         // [B][S] beam delay difference
   const int *phase0 = nullptr;          // [F][B][S] f0_f dtau[b,s] modulo one cycle, in 2^-32 cycle (from FP64)
   const float *step = nullptr;          // [B][S] fs/N * dtau[b,s], cycles per channel
-  // the same two tables with the delay compensation folded in (tensor-core plans): phase
-  // f0_f (dtau[b,s] + tau_s) reduced, step fs/N (dtau[b,s] + tau_s - n_s Ts)
-  const int *phase0g = nullptr;
+  // tensor-core plans: phase0 in cycles ([-1/2, 1/2], float) instead, and the same two tables with
+  // the delay compensation folded in: phase f0_f (dtau[b,s] + tau_s) reduced, step
+  // fs/N (dtau[b,s] + tau_s - n_s Ts)
+  const float *phase0t = nullptr;
+  const float *phase0g = nullptr;
   const float *stepg = nullptr;
   int ct16_raw = 0;           // 1: the FP16 planes hold the filtered spectrum before the delay phase
                               // and bandpass, which the tensor-core weights then carry
@@ -194,8 +196,9 @@ bool beamform_uses_split(const Geometry &g, int variant, int out_kind);
 // incoherent beam (index B of the Stokes output) from the FP32 corner-turned block
 cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct, float *out, cudaStream_t st);
 // plan-time FP64 tables of the weight phases (tables.cu)
+template <typename T>   // int: 2^-32 cycle; float: cycles
 cudaError_t launch_phase_tables(int F, int B, int S, double fs, const double *f0, const double *dtau,
-                                int *phase0, float *step, cudaStream_t st, const double *tau = nullptr,
+                                T *phase0, float *step, cudaStream_t st, const double *tau = nullptr,
                                 const double *resid = nullptr);
 // largest S the many-beam kernel accepts (shared-memory bound)
 int many_beam_max_stations();

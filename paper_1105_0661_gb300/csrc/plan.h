@@ -24,7 +24,8 @@ struct lbf_plan_s {
   float *bandpass = nullptr;
   int *dshift = nullptr;
   double *tau = nullptr, *resid = nullptr, *f0 = nullptr, *dtau = nullptr;
-  int *phase0 = nullptr, *phase0g = nullptr;
+  int *phase0 = nullptr;                        // FP32 plans
+  float *phase0t = nullptr, *phase0g = nullptr; // tensor-core plans
   float *step = nullptr;
   float *stepg = nullptr;   // with the delay folded in (tensor-core plans)
   // tensor-core precision: FP16 corner-turned planes and their TMA descriptors
@@ -66,7 +67,7 @@ struct lbf_plan_s {
     g.S = S; g.F = F; g.B = B; g.T = T; g.M = M; g.Q = Q; g.nS = nS; g.H = H; g.fs = fs;
     g.taps = taps; g.twiddle = twiddle; g.bandpass = bandpass; g.dshift = dshift;
     g.tau = tau; g.resid = resid; g.f0 = f0; g.dtau = dtau; g.phase0 = phase0; g.step = step;
-    g.phase0g = phase0g; g.stepg = stepg;
+    g.phase0t = phase0t; g.phase0g = phase0g; g.stepg = stepg;
     g.inc = inc;
     g.tc_wlo = tc_wlo;
     g.err = d_err;

@@ -149,5 +149,52 @@ __device__ __forceinline__ uint32_t pack_half2(float lo_k, float hi_k) {
   return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+// Output of short integration windows.  The lanes of an epilogue warp hold rows of windows (a row
+// per beam for I, a row per lane for IQUV: ro 0 holds I and Q, ro 1 U and V, in two buffers), but
+// each lane's row lies megabytes from the next in the output.  A warp therefore collects kW windows
+// of every row in its own piece of shared memory, the window index XORed so that neither walk meets
+// a bank twice, and writes runs of kW windows.
+template <int NS, int kW>
+struct ShortRows {
+  static constexpr int kRowsPer = 32 / kW;                        // rows per store instruction
+  static constexpr int kBuf = (NS == 1 ? 16 : 32) * kW;           // floats of one buffer
+  static constexpr int kBytes = (NS == 1 ? 1 : 2) * kBuf * 4;     // per warp
+  __device__ static int index(int row, int w) {
+    if (NS == 1) return row * kW + (w ^ ((2 * (row / kRowsPer)) & (kW - 1)));
+    return row * kW + (w ^ ((row / kRowsPer) & (kW - 1)));
+  }
+  // parameters of window w: NS 1, r0 = I (both lanes of a beam hold it); NS 4, (I, Q) or (U, V)
+  __device__ static void put(float *stage, int lane, int w, float r0, float r1) {
+    if (NS == 1) {
+      if ((w & 1) == (lane & 1)) stage[index(lane >> 1, w)] = r0;
+    } else {
+      stage[index(lane, w)] = r0;
+      stage[kBuf + index(lane, w)] = r1;
+    }
+  }
+  // windows w0 .. w0 + kW - 1 of the warp's first `nbeams` beams; row0: parameter I of the first one
+  __device__ static void flush(const float *stage, int lane, int nbeams, int w0, int Mq, float *row0, long long bstride,
+                               long long pstride) {
+    const int w = lane % kW, rl = lane / kW;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < (NS == 1 ? 16 : 32) / kRowsPer; ++k) {
+      const int row = k * kRowsPer + rl;
+      const int jq = NS == 1 ? row : row >> 1;
+      if (jq < nbeams && w0 + w < Mq) {
+        float *dst = row0 + (long long)jq * bstride + w0 + w;
+        if (NS == 1) {
+          dst[0] = stage[index(row, w)];
+        } else {
+          dst += (row & 1) * 2 * pstride;
+          dst[0] = stage[index(row, w)];
+          dst[pstride] = stage[kBuf + index(row, w)];
+        }
+      }
+    }
+    __syncwarp();   // the rows are rewritten by the next chunk
+  }
+};
+
 }  // namespace tc
 }  // namespace lbf
