@@ -457,16 +457,18 @@ cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct,
   return cudaGetLastError();
 }
 
-// The split kernel takes the many-beam forms up to 64 stations, and of the few-beam form (Stokes
-// outputs) what would be two passes or more of the few-beam kernel over enough stations: its time
-// hardly depends on the beams up to 64, the few-beam kernel's grows with passes x stations.  Measured
-// for 16 subbands of 768 spectra, Stokes I, few-beam / split: 8 stations 16 beams 0.33 / 0.40 ms and
-// 32 beams 0.66 / 0.40; 16 stations 16 beams 0.47 / 0.42; 48 stations 8 beams 0.52 / 0.59 and 16
-// beams 0.99 / 0.59; voltages of 48 stations, 16 beams (8 subbands) 0.60 / 0.94.
+// The split kernel takes the many-beam forms up to 64 stations, and of the few-beam form what would
+// be two passes or more of the few-beam kernel over enough stations: its time hardly depends on the
+// beams up to 64, the few-beam kernel's grows with passes x stations.  Measured for 768 spectra,
+// few-beam / split: Stokes I, 16 subbands: 8 stations 16 beams 0.33 / 0.33 ms, 12 stations 16 beams
+// 0.40 / 0.35, 48 stations 16 beams 0.99 / 0.53 and 8 beams 0.51 / 0.51; voltages, 8 subbands: 12
+// stations 24 beams 0.29 / 0.30, 24 stations 12 beams 0.32 / 0.33, 48 stations 9 beams 0.58 / 0.37.
+// A handful of stations over a tile of spectra is all weights: 4 stations, 64 beams, 64 spectra of 16
+// subbands 0.060 / 0.066 (many-beam kernel / split), 4 stations, 40 beams, 768 spectra 0.16 / 0.10.
 bool beamform_uses_split(const Geometry &g, int variant, int out_kind) {
   if (g.S > split_max_stations()) return false;
-  if (variant != 1) return true;
-  return out_kind != OUT_VOLTAGES && g.B > 8 && (g.B + 7) / 8 * g.S >= 24;
+  if (variant != 1) return g.S >= 8 || g.M >= 256;
+  return g.B > 8 && (g.B + 7) / 8 * g.S >= (out_kind == OUT_VOLTAGES ? 56 : 24);
 }
 
 cudaError_t launch_beamform(const Geometry &g, int variant, int out_kind, const float2 *ct, void *out,

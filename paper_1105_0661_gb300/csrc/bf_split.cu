@@ -31,20 +31,22 @@
 // An item is one UMMA M tile of 128 rows (64 beams x re|im) by the span's tiles of 64 spectra x 2
 // pols (N = 128), K = 2 stations x S padded to 16.  Warpgroup 0 holds the MMA issuer and three
 // evaluators of the next item's weights; then
-//  * converter warps (16, two groups of eight; a group owns one 32-spectrum half of each tile): each
-//    thread loads two adjacent spectra of one polarisation of every eighth station (16-byte loads,
-//    256 contiguous bytes per half-warp), the column maxima meet in shared memory across a barrier
-//    of the group, and the two slices go to the stage ring in the swizzled layout the MMA reads
-//    (32-bit stores, whole 128-byte rows: no bank conflicts).  The loads of the next tile are issued
-//    as the registers of the current one are consumed; the MMA thread prefetches the tiles after it
-//    into L2 (one tensor box per tile: a row at a time from the converters, the prefetches took
-//    2700 cycles per tile).
+//  * converter warps (8, two groups of four; a group owns one 32-spectrum half of each tile): each
+//    thread loads four adjacent spectra of one polarisation of every eighth station (one 32-byte load
+//    where rows allow it), the column maxima meet in shared memory across a barrier of the group, and
+//    the two slices go to the stage ring in the swizzled layout the MMA reads (64-bit stores, a whole
+//    128-byte row per half-warp: no bank conflicts).  The loads of the next tile are issued as the
+//    registers of the current one are consumed; the MMA thread prefetches the tiles after it into L2
+//    (one tensor box per tile: a row at a time from the converters, the prefetches took 2700 cycles
+//    per tile).  Sixteen warps of two spectra per thread: 10 % slower (twice the loop overhead).
 //  * epilogue warps (8): warp w serves TMEM lane quadrant w % 4 and one 32-spectrum half.  They take
 //    D2 into registers while the MMAs fill D1, and D1 while the MMAs fill the next tile's D2, so
 //    that one accumulator of each suffices (256 TMEM columns, next to 4 x 64 of weight slices).
-// What bounds it: the issue slots (ncu, 8 subbands of the LOFAR block: 65 % of them used), about half
-// by the converters and a fifth by the epilogue.  127 beams of the LOFAR block: 86.2 ms in FP32 FMAs,
-// 18.0 here; 37 beams of 30 subbands: 4.7 ms (five 8-beam passes) and 1.1.
+// What bounds it: the issue slots (ncu, 8 subbands of the LOFAR block: 61 % of them used, 7900 warp
+// instructions per tile of 64 beams, half of them the converters', a quarter the epilogue's) and the
+// latency of the converters' chain; the MMAs take half of a tile's 3300 cycles.  127 beams of the
+// LOFAR block: 86.2 ms in FP32 FMAs, 17.0 here; 37 beams of 30 subbands: 5.5 ms and 1.07; voltages of
+// 127 beams, 16 subbands: 5.7 ms and 1.8.
 // Every mbarrier wait is bounded: on expiry the kernel records an error code, stops issuing work,
 // waits (bounded) for its MMAs in flight, frees TMEM and returns.  The MMA thread, the evaluators and
 // the converters wait suspended; the epilogue polls (suspended waits cost it up to 70 % on short
@@ -58,7 +60,7 @@ using namespace tc;
 
 constexpr int kItemBeams = kRows / 2;       // 64 beams per work item
 constexpr int kTileSpec = 2 * kSpec;        // 64 spectra per tile
-constexpr int kEpiWarps = 8, kConvWarps = 16;
+constexpr int kEpiWarps = 8, kConvWarps = 8;
 constexpr int kGroup = kConvWarps / 2;      // converter warps per half tile
 constexpr int kThreads = 128 + 32 * (kEpiWarps + kConvWarps);   // warpgroup 0: MMA issuer (and 3 idle warps)
 constexpr int kMaxStages = 4;
@@ -80,16 +82,16 @@ constexpr uint32_t kWPlane = 64;
 constexpr float kWUnit = 128.f;
 constexpr float kMagic = 12582912.f;        // 1.5 * 2^23: x + kMagic rounds x to an integer
 constexpr int kPrefetch = 4;                // tiles an L2 prefetch runs ahead of the loads
-// registers per thread after the split of what the CTA is launched with (896 x 72 = 64512):
-// 128 x 40 + 256 x 104 + 512 x 64 = 64512
-constexpr int kLaunchRegs = 72;
+// registers per thread after the split of what the CTA is launched with (640 x 96 = 61440):
+// 128 x 40 + 256 x 120 + 256 x 96 = 60416
+constexpr int kLaunchRegs = 96;
 
 struct SpParams {
   int S, F, B, M, Kpad, ntiles, ipf;        // ipf: beam blocks per (f, c)
   int tpc, chunks;                          // tiles per item, items along the spectra
   int items, first_item;
   int stage_bytes;                          // 2 slices x 2 atoms x Kpad rows x 128 bytes
-  int vec, ctvec;                           // output rows / input rows 16-byte aligned
+  int vec, align;                           // output rows 16-byte aligned; bytes the input rows are aligned to
   const int *phase0;
   const float *step;
   const float2 *ct;
@@ -323,60 +325,27 @@ __device__ __forceinline__ void stokes_half(const float2 (&vx)[16], const float2
   }
 }
 
-// One 32-spectrum half tile as beam voltages (vol [B][F][N][P][M] cf32; `vrow0` the pol-X row of
-// the warp's first beam, beams `bstride` apart): the Re and Im lanes of a beam swap half their
-// values (one shuffle each), then 8 beams at a time go through the warp's 4 KB of shared memory
-// (spectrum index XOR 2 x beam) and leave as whole 256-byte rows.
-__device__ __forceinline__ void voltage_half(float2 (&vx)[16], float2 (&vy)[16], int m0, int ro, int jq, int lane,
-                                             int M, int B, int b0, float2 *vrow0, long long bstride, bool vec,
-                                             float2 *stage) {
-  // lane ro 0 keeps spectra 0..15 (its real parts) and gets their imaginary parts, lane ro 1 keeps
-  // 16..31: afterwards v[j] / v[8 + j] hold the complex values of spectra 16 ro + 2 j / + 1
-  auto swap = [&](float2 (&v)[16]) {
+// One 32-spectrum half tile as beam voltages (vol [B][F][N][P][M] cf32; `vrow0` the pol-X row of the
+// warp's first beam, of which `nbeams` exist, beams `bstride` apart), one polarisation at a time
+// through the warp's 4 KB: a row of 32 complex values per beam, the spectrum XORed by the beam so that
+// the 32 lanes (16 beams x re|im) write 32 banks, then out as whole 256-byte rows.
+__device__ __forceinline__ void voltage_half(const float2 (&vx)[16], const float2 (&vy)[16], int m0, int lane, int nbeams,
+                                             int M, float2 *vrow0, long long bstride, float *stage) {
+  const int ro = lane & 1, jq = lane >> 1, m = m0 + lane;
+  float *const mine = stage + jq * 64 + ro;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float2 give = ro ? v[j] : v[8 + j], keep = ro ? v[8 + j] : v[j];
-      float2 got;
-      got.x = __shfl_xor_sync(0xffffffffu, give.x, 1);
-      got.y = __shfl_xor_sync(0xffffffffu, give.y, 1);
-      v[j] = ro ? make_float2(got.x, keep.x) : make_float2(keep.x, got.x);
-      v[8 + j] = ro ? make_float2(got.y, keep.y) : make_float2(keep.y, got.y);
-    }
-  };
-  swap(vx);
-  swap(vy);
+  for (int pol = 0; pol < 2; ++pol) {
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {                // beams 8 r .. 8 r + 7 of the warp's 16
-    if ((jq >> 3) == r) {
-      const int bl = jq & 7;
-#pragma unroll
-      for (int pol = 0; pol < 2; ++pol)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          float2 *dst = stage + (bl * 2 + pol) * kSpec + 16 * ro;
-          dst[(2 * j) ^ (2 * bl)] = pol ? vy[j] : vx[j];
-          dst[(2 * j + 1) ^ (2 * bl)] = pol ? vy[8 + j] : vx[8 + j];
-        }
+    for (int i = 0; i < 16; ++i) {
+      const float2 v = pol ? vy[i] : vx[i];
+      mine[2 * ((2 * i) ^ jq)] = v.x;
+      mine[2 * ((2 * i + 1) ^ jq)] = v.y;
     }
     __syncwarp();
-    const int j2 = lane & 15;                  // spectra 2 j2, 2 j2 + 1 of the row
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int row = 2 * k + (lane >> 4);     // (beam, pol) of the 8 staged beams
-      const int bl = row >> 1, pol = row & 1;
-      const int s0 = 2 * j2;
-      const float4 val = *reinterpret_cast<const float4 *>(stage + row * kSpec + (s0 & 16) + ((s0 & 15) ^ (2 * bl)));
-      const int m = m0 + s0;
-      if (b0 + 8 * r + bl < B) {
-        float2 *dst = vrow0 + (long long)(8 * r + bl) * bstride + (long long)pol * M + m;
-        if (vec && m + 1 < M) {
-          *reinterpret_cast<float4 *>(dst) = val;
-        } else {
-          if (m < M) dst[0] = make_float2(val.x, val.y);
-          if (m + 1 < M) dst[1] = make_float2(val.z, val.w);
-        }
-      }
-    }
+    float2 *dst = vrow0 + (long long)pol * M + m;
+#pragma unroll 8
+    for (int b = 0; b < 16; ++b, dst += bstride)
+      if (b < nbeams && m < M) *dst = *reinterpret_cast<const float2 *>(stage + b * 64 + 2 * (lane ^ b));
     __syncwarp();
   }
 }
@@ -456,29 +425,37 @@ __device__ __forceinline__ bool group_sync_any(uint32_t id, uint32_t n, bool pre
   return r != 0;
 }
 
-// Four consecutive floats (two spectra) of a corner-turned row into v, which keeps its value where
-// nothing is loaded (`one`, `two`: the first and the second spectrum exist).
-template <bool kVec>
-__device__ __forceinline__ void load_pair(float4 &v, const float2 *p, bool one, bool two) {
-  if constexpr (kVec) {
+// Four consecutive spectra (32 bytes) of a corner-turned row into v, which keeps its value where
+// nothing is loaded: n spectra exist from p on.  kAl: bytes the rows are aligned to.
+template <int kAl>
+__device__ __forceinline__ void load_quad(float (&v)[8], const float2 *p, int n) {
+  if constexpr (kAl == 32) {   // four spectra or none
     asm volatile(
-        "{\n\t.reg .pred a;\n\tsetp.ne.u32 a, %5, 0;\n\t"
-        "@a ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
-        : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
-        : "l"(p), "r"((uint32_t)one));
+        "{\n\t.reg .pred a;\n\tsetp.gt.s32 a, %9, 0;\n\t"
+        "@a ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t}"
+        : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])
+        : "l"(p), "r"(n));
+  } else if constexpr (kAl == 16) {   // an even number
+    asm volatile(
+        "{\n\t.reg .pred a, b;\n\tsetp.gt.s32 a, %9, 0;\n\tsetp.gt.s32 b, %9, 2;\n\t"
+        "@a ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%8];\n\t"
+        "@b ld.global.nc.v4.f32 {%4, %5, %6, %7}, [%8+16];\n\t}"
+        : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])
+        : "l"(p), "r"(n));
   } else {
     asm volatile(
-        "{\n\t.reg .pred a, b;\n\tsetp.ne.u32 a, %5, 0;\n\tsetp.ne.u32 b, %6, 0;\n\t"
-        "@a ld.global.nc.v2.f32 {%0, %1}, [%4];\n\t"
-        "@b ld.global.nc.v2.f32 {%2, %3}, [%4+8];\n\t}"
-        : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
-        : "l"(p), "r"((uint32_t)one), "r"((uint32_t)two));
+        "{\n\t.reg .pred a, b, c, d;\n\tsetp.gt.s32 a, %9, 0;\n\tsetp.gt.s32 b, %9, 1;\n\t"
+        "setp.gt.s32 c, %9, 2;\n\tsetp.gt.s32 d, %9, 3;\n\t"
+        "@a ld.global.nc.v2.f32 {%0, %1}, [%8];\n\t@b ld.global.nc.v2.f32 {%2, %3}, [%8+8];\n\t"
+        "@c ld.global.nc.v2.f32 {%4, %5}, [%8+16];\n\t@d ld.global.nc.v2.f32 {%6, %7}, [%8+24];\n\t}"
+        : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])
+        : "l"(p), "r"(n));
   }
 }
 
 // The converter role.  NLD: stations per thread (at least Kpad / 16), so that a tile's loads are
 // straight-line code: behind a branch per station they ran one after the other (7000 cycles per tile).
-template <int NLD, bool kVec, bool kMulti>
+template <int NLD, int kAl, bool kMulti>
 __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const sbase, int cw, int lane) {
   const uint32_t bar0 = smem_u32(sbase);
   float *const scales = reinterpret_cast<float *>(sbase + kScaleOff);
@@ -489,11 +466,13 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 64u + 8u * s; };
   const int grp = cw / kGroup, wg = cw % kGroup;
-  const int pol = lane >> 4, j = lane & 15;
-  const int col = grp * kSpec + 2 * j;        // first spectrum of the thread within a tile
-  float4 r[NLD];                              // two spectra of every eighth station
+  const int s0 = 2 * wg + (lane >> 4);       // station within a step of 2 kGroup
+  const int pol = (lane >> 3) & 1, j = lane & 7;
+  const int col = grp * kSpec + 4 * j;       // first spectrum of the thread within a tile
+  const int cc = pol * kSpec + 4 * j;        // its first column within the half tile
+  float r[NLD][8];                            // four spectra of every eighth station
   int item = blockIdx.x, t = 0, t1 = 0, pi = 0;
-  const float2 *ptr = nullptr;                // row of station wg, at this thread's spectrum of the tile
+  const float2 *ptr = nullptr;                // row of station s0, at this thread's spectra of the tile
   auto plan = [&]() -> const SpParams & { return L.plan[kMulti ? pi : 0]; };
   auto enter = [&]() {
     if (kMulti) pi = plan_of(L, item);
@@ -501,53 +480,50 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
     const Item w = item_of(p, item);
     t = w.t0;
     t1 = w.t1;
-    ptr = p.ct + (((long long)w.fc * p.S + wg) * kP + pol) * p.M + t * kTileSpec + col;
+    ptr = p.ct + (((long long)w.fc * p.S + s0) * kP + pol) * p.M + t * kTileSpec + col;
   };
-  // Station wg + 8 i of the first S.  Pad stations keep finite values, which meet weights of zero;
+  // Station s0 + 8 i of the first S.  Pad stations keep finite values, which meet weights of zero;
   // columns past M keep what they held and are never stored.
   auto load_tile = [&](int i, int S, int M) {
-    const bool in = wg + kGroup * i < S;
-    const int m = t * kTileSpec + col;
-    load_pair<kVec>(r[i], ptr + (long long)(i * kGroup * kP) * M, in && m < M, in && m + 1 < M);
+    load_quad<kAl>(r[i], ptr + (long long)(i * 2 * kGroup * kP) * M, s0 + 2 * kGroup * i < S ? M - (t * kTileSpec + col) : 0);
   };
-  auto clear = [&]() {
+  auto clear = [&](int i) {
 #pragma unroll
-    for (int i = 0; i < NLD; ++i) r[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int e = 0; e < 8; ++e) r[i][e] = 0.f;
   };
-  clear();
+#pragma unroll
+  for (int i = 0; i < NLD; ++i) clear(i);
   enter();
   {
     const int S = plan().S, M = plan().M;
 #pragma unroll
     for (int i = 0; i < NLD; ++i) load_tile(i, S, M);
   }
-  if (wg == 0) colmax[grp * 3 * 64 + 2 * lane] = colmax[grp * 3 * 64 + 2 * lane + 1] = 0;   // n = 0
+  uint32_t *const cm0 = colmax + grp * 3 * 64;
+  if (wg == 0) cm0[2 * lane] = cm0[2 * lane + 1] = 0;   // n = 0
   group_sync_any(1 + grp, 32 * kGroup, false);
   int s = 0, slot = 0, n = 0;
   uint32_t ph = 0;
   int b3 = 0;
   bool failed = false, more = true;
   while (more) {
-    const SpParams &p = plan();
-    const int Kpad = p.Kpad;
-    float f0 = 0.f, f1 = 0.f;                 // largest component of the two columns (NaNs ignored)
+    const int Kpad = plan().Kpad;
+    float mx[4] = {0.f, 0.f, 0.f, 0.f};       // largest component of the four columns (NaNs ignored)
 #pragma unroll
-    for (int i = 0; i < NLD; ++i) {
-      f0 = fmaxf(f0, fmaxf(fabsf(r[i].x), fabsf(r[i].y)));
-      f1 = fmaxf(f1, fmaxf(fabsf(r[i].z), fabsf(r[i].w)));
-    }
+    for (int i = 0; i < NLD; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) mx[e] = fmaxf(mx[e], fmaxf(fabsf(r[i][2 * e]), fabsf(r[i][2 * e + 1])));
     // three rotating maxima per column: tile n's, tile n + 1's cleared before the barrier (its
     // readers, of tile n - 2, passed the barrier of tile n - 1)
-    uint32_t *cm = colmax + (grp * 3 + b3) * 64 + 2 * lane;
+    uint32_t *cm = cm0 + b3 * 64 + pol * 8 + j;   // [4 columns of a thread][16 threads]
     b3 = b3 == 2 ? 0 : b3 + 1;
-    atomicMax(cm, __float_as_uint(f0));
-    atomicMax(cm + 1, __float_as_uint(f1));
-    if (wg == 0) *reinterpret_cast<uint2 *>(colmax + (grp * 3 + b3) * 64 + 2 * lane) = make_uint2(0, 0);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) atomicMax(cm + 16 * e, __float_as_uint(mx[e]));
+    if (wg == 0) *reinterpret_cast<uint2 *>(cm0 + b3 * 64 + 2 * lane) = make_uint2(0, 0);
     if (failed) gfail[grp * 2 + (n & 1)] = 1;
-    const bool inf = group_sync_any(1 + grp, 32 * kGroup, fmaxf(f0, f1) > 3.402823466e38f);
+    const bool inf = group_sync_any(1 + grp, 32 * kGroup,
+                                    fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) > 3.402823466e38f);
     if (gfail[grp * 2 + (n & 1)]) break;      // the whole group leaves together
-    const uint2 cc = *reinterpret_cast<const uint2 *>(cm);
-    const uint32_t c0 = cc.x, c1 = cc.y;
     // scale 2^(137 - E) for a peak in [2^(E - 127), 2^(E - 126)): the peak lands in [2^10, 2^11);
     // its inverse, with the weights' 2^7, is 2^(E - 144) (subnormal for E < 18)
     auto scale_of = [](uint32_t cb, float &inv) {
@@ -555,17 +531,18 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
       inv = E >= 18 ? __uint_as_float((uint32_t)(E - 17) << 23) : __uint_as_float(1u << (E + 5));
       return __uint_as_float((uint32_t)(264 - min(E, 254)) << 23);
     };
-    float i0, i1;
-    const float s0 = scale_of(c0, i0), s1 = scale_of(c1, i1);
-    if (!mbar_wait_suspended(empty_bar(s), ph ^ 1u, abort_flag)) { fail(abort_flag, p.err, ERR_PRODUCER); failed = true; }
+    float4 inv;
+    const float sc[4] = {scale_of(cm[0], inv.x), scale_of(cm[16], inv.y), scale_of(cm[32], inv.z),
+                         scale_of(cm[48], inv.w)};
+    if (!mbar_wait_suspended(empty_bar(s), ph ^ 1u, abort_flag)) { fail(abort_flag, plan().err, ERR_PRODUCER); failed = true; }
     // row k of a slice's atom: 128 bytes [pol X | pol Y][32 spectra], 16-byte chunks XOR (k & 7);
-    // station wg + 8 i holds rows k = 2 wg + 16 i (re) and k + 1 (im).  (After an expired wait the
+    // station s0 + 8 i holds rows k = 2 s0 + 16 i (re) and k + 1 (im).  (After an expired wait the
     // stage is overwritten all the same: the launch has failed.)
-    unsigned char *hi0 = sbase + kRingOff + (size_t)s * L.stage_max + (size_t)grp * (Kpad * 128);
-    const uint32_t chunk = (uint32_t)(pol * 4 + (j >> 2)), within = (uint32_t)(j & 3) * 4;
-    const int k0 = 2 * wg;
-    unsigned char *re = hi0 + k0 * 128 + ((chunk ^ (uint32_t)(k0 & 7)) << 4) + within;
-    unsigned char *im = hi0 + (k0 + 1) * 128 + ((chunk ^ (uint32_t)((k0 + 1) & 7)) << 4) + within;
+    const uint32_t chunk = (uint32_t)(pol * 4 + (j >> 1)), within = (uint32_t)(j & 1) * 8;
+    const int k0 = 2 * s0;
+    unsigned char *re = sbase + kRingOff + (size_t)s * L.stage_max + (size_t)grp * (Kpad * 128) + k0 * 128 + within;
+    unsigned char *im = re + 128 + ((chunk ^ (uint32_t)((k0 + 1) & 7)) << 4);
+    re += (chunk ^ (uint32_t)(k0 & 7)) << 4;
     const uint32_t lo_off = (uint32_t)Kpad * 256;
     // on to the next tile
     ptr += kTileSpec;
@@ -575,28 +552,28 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
       if (more) enter();
     }
     const int nS = more ? plan().S : 0, nM = plan().M;
-    const float2 sa = make_float2(s0, s0), sb = make_float2(s1, s1), mg = make_float2(kMagic, kMagic);
-    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 mg = make_float2(kMagic, kMagic), m1 = make_float2(-1.f, -1.f);
 #pragma unroll
     for (int i = 0; i < NLD; ++i) {
-      const float2 a = make_float2(r[i].x, r[i].y), b = make_float2(r[i].z, r[i].w);
-      const float2 ta = __ffma2_rn(a, sa, mg), tb = __ffma2_rn(b, sb, mg);      // integers + kMagic
-      const float2 ha = __ffma2_rn(ta, m1, mg), hb = __ffma2_rn(tb, m1, mg);    // minus the leading slice
-      const float2 la = __ffma2_rn(a, sa, ha), lb = __ffma2_rn(b, sb, hb);
-      if (k0 + 2 * kGroup * i < Kpad) {
-        *reinterpret_cast<uint32_t *>(re + i * (kGroup * 256)) = pack_half2(-ha.x, -hb.x);
-        *reinterpret_cast<uint32_t *>(im + i * (kGroup * 256)) = pack_half2(-ha.y, -hb.y);
-        *reinterpret_cast<uint32_t *>(re + lo_off + i * (kGroup * 256)) = pack_half2(la.x, lb.x);
-        *reinterpret_cast<uint32_t *>(im + lo_off + i * (kGroup * 256)) = pack_half2(la.y, lb.y);
+      float2 h[4], l[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 x = make_float2(r[i][2 * e], r[i][2 * e + 1]), sx = make_float2(sc[e], sc[e]);
+        h[e] = __ffma2_rn(__ffma2_rn(x, sx, mg), m1, mg);   // minus the leading slice
+        l[e] = __ffma2_rn(x, sx, h[e]);
       }
-      if (kMulti) r[i] = make_float4(0.f, 0.f, 0.f, 0.f);   // the next plan may have fewer stations
+      if (k0 + 4 * kGroup * i < Kpad) {
+        *reinterpret_cast<uint2 *>(re + i * (kGroup * 512)) = make_uint2(pack_half2(-h[0].x, -h[1].x), pack_half2(-h[2].x, -h[3].x));
+        *reinterpret_cast<uint2 *>(im + i * (kGroup * 512)) = make_uint2(pack_half2(-h[0].y, -h[1].y), pack_half2(-h[2].y, -h[3].y));
+        *reinterpret_cast<uint2 *>(re + lo_off + i * (kGroup * 512)) = make_uint2(pack_half2(l[0].x, l[1].x), pack_half2(l[2].x, l[3].x));
+        *reinterpret_cast<uint2 *>(im + lo_off + i * (kGroup * 512)) = make_uint2(pack_half2(l[0].y, l[1].y), pack_half2(l[2].y, l[3].y));
+      }
+      if (kMulti) clear(i);                   // the next plan may have fewer stations
       load_tile(i, nS, nM);
     }
     if (!failed) {
-      if (wg == 0) {
-        *reinterpret_cast<float2 *>(scales + slot * kCols + grp * 64 + 2 * lane) = make_float2(i0, i1);
-        if (lane == 0) nonfinite[slot * 2 + grp] = inf ? 1 : 0;
-      }
+      if (wg == 0 && lane < 16) *reinterpret_cast<float4 *>(scales + slot * kCols + grp * 64 + cc) = inv;
+      if (wg == 0 && lane == 0) nonfinite[slot * 2 + grp] = inf ? 1 : 0;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the slices visible to the MMA
       __syncwarp();
       if (lane == 0) mbar_arrive(full_bar(s));
@@ -673,7 +650,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
       uint32_t ph = 0, gpar = 0;
       int *err = L.plan[0].err;
       // the tile kPrefetch tiles on goes to L2 (one box of all its rows) while the MMAs run
-      const bool pf = !kMulti && L.plan[0].ctvec;
+      const bool pf = !kMulti && L.plan[0].align >= 16;
       int pitem = blockIdx.x, pt = 0, pt1 = 0, pfc = 0;
       auto prefetch = [&](bool fetch) {
         if (pitem >= L.items) return;
@@ -743,7 +720,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
     }
     __syncwarp();
   } else if (warp < 4 + kEpiWarps) {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
     // ---------------------------------------------------------------- epilogue
     const int ew = warp - 4, quad = warp & 3, half = ew >> 2;
     const int ro = lane & 1, jq = lane >> 1;
@@ -844,8 +821,8 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
         float *const buf = qbuf + (fl & 1) * St::kBuf;
         if constexpr (NS == 0) {
           float2 *const v0 = reinterpret_cast<float2 *>(p.out) + (((long long)b0 * p.F + f) * kN + c) * kP * p.M;
-          voltage_half(vx, vy, m0, ro, jq, lane, p.M, p.B, b0, v0, (long long)p.F * kN * kP * p.M, p.vec != 0,
-                       reinterpret_cast<float2 *>(stage_out) + ew * (kVStageBytes / 8));
+          voltage_half(vx, vy, m0, lane, nb, p.M, v0, (long long)p.F * kN * kP * p.M,
+                       stage_out + ew * (kVStageBytes / 4));
         } else {
           stokes_half<NS, Q>(vx, vy, m0, lane, nb, p.M, row0, NS * pstride, pstride, buf + jq * St::kRow,
                              stage_out + ew * (kVStageBytes / 4), wbase);
@@ -872,14 +849,14 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
     }
   } else {
     // ---------------------------------------------------------------- converters
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     const int cw = warp - 4 - kEpiWarps;
-    const int nld = L.plan[0].Kpad / 16;
-    if (kMulti || !L.plan[0].ctvec) convert<8, false, kMulti>(L, sbase, cw, lane);
-    else if (nld <= 2) convert<2, true, kMulti>(L, sbase, cw, lane);
-    else if (nld <= 4) convert<4, true, kMulti>(L, sbase, cw, lane);
-    else if (nld <= 6) convert<6, true, kMulti>(L, sbase, cw, lane);
-    else convert<8, true, kMulti>(L, sbase, cw, lane);
+    const int nld = L.plan[0].Kpad / 16, al = L.plan[0].align;
+    if (kMulti || al == 8) convert<8, 8, kMulti>(L, sbase, cw, lane);
+    else if (al == 16) convert<8, 16, kMulti>(L, sbase, cw, lane);
+    else if (nld <= 2) convert<2, 32, kMulti>(L, sbase, cw, lane);
+    else if (nld <= 4) convert<4, 32, kMulti>(L, sbase, cw, lane);
+    else if (nld <= 6) convert<6, 32, kMulti>(L, sbase, cw, lane);
+    else convert<8, 32, kMulti>(L, sbase, cw, lane);
   }
 
   tc_fence_before();
@@ -964,8 +941,9 @@ bool fill_plan(SpLaunch &L, int i, const Geometry &g, int out_kind, const float2
   p.err = g.err;
   const bool aligned = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
   p.vec = aligned && (out_kind == OUT_VOLTAGES ? g.M % 2 == 0 : (g.M / g.Q) % 4 == 0);
-  p.ctvec = g.M % 2 == 0 && (reinterpret_cast<uintptr_t>(ct) & 15) == 0;
-  if (p.ctvec && encode_ct32_tile_map(&L.map[i], ct, 2 * g.S, g.M, (long long)g.F * kN, kTileSpec) != cudaSuccess)
+  const uintptr_t ca = reinterpret_cast<uintptr_t>(ct);
+  p.align = g.M % 4 == 0 && (ca & 31) == 0 ? 32 : g.M % 2 == 0 && (ca & 15) == 0 ? 16 : 8;
+  if (p.align >= 16 && encode_ct32_tile_map(&L.map[i], ct, 2 * g.S, g.M, (long long)g.F * kN, kTileSpec) != cudaSuccess)
     return false;
   L.items = p.first_item + p.items;
   L.stage_max = p.stage_bytes > L.stage_max ? p.stage_bytes : L.stage_max;
