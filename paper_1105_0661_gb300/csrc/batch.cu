@@ -61,7 +61,7 @@ struct lbf_batch_s {
                                                       // ppf_group_maps_bytes()), pinned host / device
   lbf::BfGroup *h_bf = nullptr;                      // pinned host, 2 * n: FP32 plans, class by class
   unsigned long long *d_counter = nullptr;            // [max_counters(n)] work counters, one per launch
-  long long hist_items = 0;
+  long long hist_streams = 0;
   // launch classes: filter bank per (sample width, FP32 or FP16 output); FP32 beam former per
   // (variant, output kind, CTAs per SM) -- each class one persistent launch over its groups
   struct PpfClass { int bits, tc, tma, first, n; long long items; };
@@ -97,7 +97,7 @@ long long tc_class(const lbf_plan_s *p) {
 
 // Fill the group tables of parity `par` (par = 1: every plan's history one block ahead) for the
 // given block buffers: filter-bank groups class by class (work items numbered from 0 within a
-// class; history elements numbered over the whole table), then the FP32 beam-former groups class
+// class; history streams numbered over the whole table), then the FP32 beam-former groups class
 // by class.
 void fill_tables(lbf_batch_t b, int par, const void *const *d_in, void *const *d_out) {
   const int n = (int)b->plans.size();
@@ -137,17 +137,17 @@ void fill_tables(lbf_batch_t b, int par, const void *const *d_in, void *const *d
         G.spc = b->spc;
         G.chunks = lbf::ppf_items_per_stream(p->M, b->spc);
         G.first_item = cls.items;
-        G.first_hist = hi;
+        G.first_stream = hi;
         G.maps = nullptr;
         if (tma && lbf::ppf_group_maps(G, b->h_maps + (size_t)at * mb) == cudaSuccess)
           G.maps = b->d_maps + (size_t)at * mb;
         cls.items += (long long)p->S * p->F * G.chunks;   // one item: both polarisations of a chunk
-        hi += (long long)p->S * p->F * p->H;
+        hi += (long long)p->S * p->F;
         ++cls.n;
       }
       if (cls.n) b->ppf_cls.push_back(cls);
     }
-  b->hist_items = hi;
+  b->hist_streams = hi;
   b->tc_out.assign(d_out, d_out + n);
   b->d_in_cur.assign(d_in, d_in + n);
   // FP32 beam former: plans of the same variant, output kind and residency share a launch
@@ -156,7 +156,7 @@ void fill_tables(lbf_batch_t b, int par, const void *const *d_in, void *const *d
   for (int i = 0; i < n; ++i) {
     lbf_plan_t p = b->plans[i];
     if (p->tc || split_plan(b, i)) continue;
-    smem_of[i] = lbf::bf_smem_bytes(b->variant[i], p->S);
+    smem_of[i] = lbf::bf_smem_bytes(b->variant[i], p->S, p->M);
     per_sm[i] = lbf::bf_group_residency(b->variant[i], p->out_kind, smem_of[i]);
   }
   b->bf_cls.clear();
@@ -179,9 +179,10 @@ void fill_tables(lbf_batch_t b, int par, const void *const *d_in, void *const *d
       Bg.variant = b->variant[j];
       Bg.out_kind = p->out_kind;
       const int per = b->variant[j] == 1 ? lbf::few_beams_per_item() : lbf::many_beams_per_item(b->variant[j]);
+      Bg.lg = b->variant[j] == 1 ? lbf::few_log_channels(p->M, p->S) : 0;
       Bg.per_fc = (p->B + per - 1) / per;
       Bg.first_item = cls.items;
-      cls.items += (long long)p->F * lbf::kN * Bg.per_fc;
+      cls.items += (((long long)p->F * lbf::kN) >> Bg.lg) * Bg.per_fc;
       cls.smem = smem_of[j] > cls.smem ? smem_of[j] : cls.smem;
       ++cls.n;
     }
@@ -201,7 +202,7 @@ cudaError_t enqueue(lbf_batch_t b, int par, cudaStream_t st) {
     e = cudaMemcpyAsync(b->d_maps + (size_t)par * n * mb, b->h_maps + (size_t)par * n * mb, mb * n,
                         cudaMemcpyHostToDevice, st);
   if (b->per_plan) {
-    // each plan's own filter bank, history update and FP32 beam former (the hardware schedules
+    // each plan's own filter bank (and history) and FP32 beam former (the hardware schedules
     // their CTAs; large observations each fill the GPU); the tensor-core plans follow, one
     // launch each
     for (int i = 0; i < n && e == cudaSuccess; ++i) {
@@ -210,16 +211,18 @@ cudaError_t enqueue(lbf_batch_t b, int par, cudaStream_t st) {
       const int cur = p->cur ^ par;
       const lbf::Geometry g = p->geometry();
       const void *din = b->d_in_cur[i];
+      const bool fused = lbf::ppf_fuses_history(g);
       if (p->tc) {
         lbf::Ct16Out o;
         o.hi = p->ct16[0];
         o.lo = static_cast<unsigned char *>(p->ct16[0]) + p->ct16_bytes;
         o.kpad = p->kpad;
-        e = lbf::launch_ppf(g, p->bits, din, p->hist[cur], nullptr, nullptr, st, &o);
+        e = lbf::launch_ppf(g, p->bits, din, p->hist[cur], fused ? p->hist[cur ^ 1] : nullptr, nullptr, nullptr, st, &o);
       } else {
-        e = lbf::launch_ppf(g, p->bits, din, p->hist[cur], nullptr, p->ws, st);
+        e = lbf::launch_ppf(g, p->bits, din, p->hist[cur], fused ? p->hist[cur ^ 1] : nullptr, nullptr, p->ws, st);
       }
-      if (e == cudaSuccess) e = lbf::launch_hist_update(g, p->bits, din, p->hist[cur], p->hist[cur ^ 1], st);
+      if (e == cudaSuccess && !fused)
+        e = lbf::launch_hist_update(g, p->bits, din, p->hist[cur], p->hist[cur ^ 1], st);
       if (e == cudaSuccess && !p->tc) e = lbf::launch_beamform(g, b->variant[i], p->out_kind, p->ws, b->tc_out[i], st);
     }
   } else {
@@ -229,7 +232,7 @@ cudaError_t enqueue(lbf_batch_t b, int par, cudaStream_t st) {
       if (e == cudaSuccess)
         e = lbf::launch_ppf_group(c.bits, c.tc, c.tma, b->h_ppf + par * n + c.first, c.n, c.items,
                                   b->d_counter + counter++, b->ppf_ctas, st);
-    if (e == cudaSuccess) e = lbf::launch_hist_group(b->d_ppf + par * n, n, b->hist_items, st);
+    if (e == cudaSuccess) e = lbf::launch_hist_group(b->d_ppf + par * n, n, b->hist_streams, st);
     for (const auto &c : b->bf_cls)
       if (e == cudaSuccess)
         e = lbf::launch_bf_group(c.variant, c.out_kind, b->h_bf + par * n + c.first, c.n, c.items,
@@ -412,11 +415,11 @@ lbf_status lbf_batch_launches(lbf_batch_t b, int32_t *n_launches) {
   if (!b || b->magic != kBatchMagic) return LBF_ESTATE;
   if (!n_launches) return LBF_EINVAL;
   // classes of the tables last filled (lbf_batch_run, lbf_batch_capture or lbf_batch_tune)
-  if (b->per_plan) {   // per plan: filter bank, history and beam former (+ incoherent beam) each
+  if (b->per_plan) {   // per plan: filter bank (+ history) and beam former (+ incoherent beam) each
     int k = 0;
     for (size_t i = 0; i < b->plans.size(); ++i) {
       lbf_plan_t p = b->plans[i];
-      k += p->M ? 3 + (p->inc && (p->tc || split_plan(b, (int)i)) ? 1 : 0) : 0;
+      k += p->M ? (lbf::ppf_fuses_history(p->geometry()) ? 2 : 3) + (p->inc && (p->tc || split_plan(b, (int)i)) ? 1 : 0) : 0;
     }
     *n_launches = k;
     return LBF_OK;

@@ -65,15 +65,22 @@ struct IncAcc {
 };
 
 // ------------------------------------------------------------------------------- few beams
-// Work item: (subband, channel) fc, beams bgrp * FB .. + FB - 1.  FB = 16 reads the corner-turned
-// block half as often for 9 to 32 beams (16 FP32 flop per byte, about the FP32/HBM ridge).
-template <int OUT, int FB = kFewBeams>
+// Work item: 2^lg channels from (subband, channel) fc0 << lg on, beams bgrp * FB .. + FB - 1; 256 >> lg
+// threads (whole warps) take each channel's spectra, so that blocks of up to 128 spectra fill the CTA
+// (few_log_channels).  FB = 16 reads the corner-turned block half as often for 9 to 32 beams (16 FP32
+// flop per byte, about the FP32/HBM ridge).
+// kOne: lg is 0 (known to the compiler, which then keeps the item's pointers in uniform registers).
+template <int OUT, int FB, bool kOne>
 __device__ __forceinline__ void bf_few_item(const Geometry &g, const float2 *__restrict__ ct, void *__restrict__ out,
-                                            int fc, int bgrp, float2 *wsm /* [S][FB] */) {
-  const int f = fc / kN, c = fc - f * kN;
+                                            int fc0, int lg, int bgrp, float2 *wsm /* [2^lg][S][FB] */) {
   const int b0 = bgrp * FB;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < g.S * FB; i += kFewThreads) {
+  const int lt = kOne ? 8 : 8 - lg;           // log2 of the threads of a channel
+  const int tid = kOne ? threadIdx.x : threadIdx.x & ((1 << lt) - 1);
+  const int sub = kOne ? 0 : __shfl_sync(0xffffffffu, threadIdx.x >> lt, 0);
+  const int fc = kOne ? fc0 : (fc0 << lg) + sub;
+  const int f = fc / kN, c = fc - f * kN;     // (the item's channels lie in one subband)
+  wsm += sub * g.S * FB;
+  for (int i = tid; i < g.S * FB; i += 1 << lt) {
     const int s = i / FB, b = b0 + (i - s * FB);
     wsm[i] = (b < g.B) ? beam_weight(g, f, c, (long long)b * g.S + s) : make_float2(0.f, 0.f);
   }
@@ -81,7 +88,7 @@ __device__ __forceinline__ void bf_few_item(const Geometry &g, const float2 *__r
   const float2 *y = ct + (long long)fc * g.S * kP * g.M;
   const int nS = (OUT == OUT_STOKES_IQUV) ? 4 : 1;
   const int Mq = g.M / g.Q;
-  for (int mb = 0; mb < g.M; mb += kFewThreads) {
+  for (int mb = 0; mb < g.M; mb += 1 << lt) {
     const int m = mb + tid;
     const bool active = m < g.M;
     float2 acc[FB][kP];
@@ -148,27 +155,38 @@ __device__ __forceinline__ void bf_few_item(const Geometry &g, const float2 *__r
 // at least two CTAs per SM (three for the 8-beam Stokes I form): a bandwidth-bound kernel needs
 // the warps; left to itself the compiler gave the IQUV form 194 registers, one CTA per SM and 2.6x
 // the Stokes I time
-template <int OUT, int FB>
+template <int OUT, int FB, bool kOne>
 __global__ void __launch_bounds__(kFewThreads, (OUT == OUT_STOKES_I && FB == 8) ? 3 : 2)
-bf_few_kernel(Geometry g, const float2 *__restrict__ ct, void *__restrict__ out) {
+bf_few_kernel(Geometry g, const float2 *__restrict__ ct, void *__restrict__ out, int lg) {
   extern __shared__ __align__(16) float2 wsm[];
-  bf_few_item<OUT, FB>(g, ct, out, blockIdx.x, blockIdx.y, wsm);
+  bf_few_item<OUT, FB, kOne>(g, ct, out, blockIdx.x, lg, blockIdx.y, wsm);
+}
+
+// Channels per work item of the few-beam kernel, as a power of two: as many as fill its 256 threads
+// with whole warps of spectra, within 48 KB of weights.  64 observations of 64 spectra (8-16
+// stations, 1-8 beams, grouped): one channel per item 1.29 ms, four 0.43 ms.
+int few_log_channels(int M, int S, int FB) {
+  int lg = M <= 32 ? 3 : M <= 64 ? 2 : M <= 128 ? 1 : 0;
+  while (lg > 0 && ((size_t)S * FB * sizeof(float2) << lg) > 48 * 1024) --lg;
+  return lg;
 }
 
 template <int FB>
 cudaError_t launch_few(const Geometry &g, int out_kind, const float2 *ct, void *out, cudaStream_t st) {
-  dim3 grid((unsigned)(g.F * kN), (unsigned)((g.B + FB - 1) / FB));
-  const size_t smem = (size_t)g.S * FB * sizeof(float2);
+  const int fb = out_kind == OUT_STOKES_I ? FB : 8;
+  const int lg = few_log_channels(g.M, g.S, fb);
+  dim3 grid((unsigned)((g.F * kN) >> lg), (unsigned)((g.B + fb - 1) / fb));
+  const size_t smem = ((size_t)g.S * fb * sizeof(float2)) << lg;
   auto go = [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kFewThreads, smem, st>>>(g, ct, out);
+    kern<<<grid, kFewThreads, smem, st>>>(g, ct, out, lg);
     return cudaGetLastError();
   };
   switch (out_kind) {
-    case OUT_VOLTAGES: return go(bf_few_kernel<OUT_VOLTAGES, 8>);
-    case OUT_STOKES_I: return go(bf_few_kernel<OUT_STOKES_I, FB>);
-    default: return go(bf_few_kernel<OUT_STOKES_IQUV, 8>);
+    case OUT_VOLTAGES: return lg ? go(bf_few_kernel<OUT_VOLTAGES, 8, false>) : go(bf_few_kernel<OUT_VOLTAGES, 8, true>);
+    case OUT_STOKES_I: return lg ? go(bf_few_kernel<OUT_STOKES_I, FB, false>) : go(bf_few_kernel<OUT_STOKES_I, FB, true>);
+    default: return lg ? go(bf_few_kernel<OUT_STOKES_IQUV, 8, false>) : go(bf_few_kernel<OUT_STOKES_IQUV, 8, true>);
   }
 }
 
@@ -398,7 +416,10 @@ bf_group_kernel(const __grid_constant__ BfTable T, long long total, unsigned lon
     const BfGroup &G = T.grp[o];
     const long long local = item - G.first_item;
     const int fc = (int)(local / G.per_fc), sub = (int)(local - (long long)fc * G.per_fc);
-    if constexpr (V == 1) bf_few_item<OUT>(G.g, G.ct, G.out, fc, sub, smem);
+    if constexpr (V == 1) {
+      if (G.lg == 0) bf_few_item<OUT, kFewBeams, true>(G.g, G.ct, G.out, fc, 0, sub, smem);
+      else bf_few_item<OUT, kFewBeams, false>(G.g, G.ct, G.out, fc, G.lg, sub, smem);
+    }
     else if constexpr (V == 3) bf_many_item<OUT, 64>(G.g, G.ct, G.out, fc, sub, smem);
     else bf_many_item<OUT, 128>(G.g, G.ct, G.out, fc, sub, smem);
   }
@@ -565,8 +586,9 @@ int bf_group_residency(int variant, int out_kind, size_t smem) {
 
 int few_beams_per_item() { return kFewBeams; }
 int many_beams_per_item(int variant) { return variant == 3 ? 64 : kBT; }
-size_t bf_smem_bytes(int variant, int S) {
-  if (variant == 1) return (size_t)S * kFewBeams * sizeof(float2);
+int few_log_channels(int M, int S) { return few_log_channels(M, S, kFewBeams); }
+size_t bf_smem_bytes(int variant, int S, int M) {
+  if (variant == 1) return ((size_t)S * kFewBeams * sizeof(float2)) << few_log_channels(M, S, kFewBeams);
   return (size_t)S * ((variant == 3 ? 64 : kBT) + 2 * kP * kMC) * sizeof(float2);
 }
 

@@ -251,6 +251,19 @@ void trace_free(lbf_plan_t p) {
 
 int bf_kernel_id(lbf_plan_t p) { return p->variant == 1 ? K_BF_FEW : p->variant == 3 ? K_BF_MANY64 : K_BF_MANY; }
 
+// The filter bank of one block with the next block's history, in one launch or two.
+cudaError_t filter_bank(lbf_plan_t p, int kernel, const lbf::Geometry &g, const void *d_in, float2 *chan, float2 *ct,
+                        const lbf::Ct16Out *o, cudaStream_t st) {
+  const void *h = p->hist[p->cur];
+  void *nh = p->hist[p->cur ^ 1];
+  const bool fused = lbf::ppf_fuses_history(g);
+  cudaError_t e = traced(p, kernel, st, [&] {
+    return lbf::launch_ppf(g, p->bits, d_in, h, fused ? nh : nullptr, chan, ct, st, o); });
+  if (e == cudaSuccess && !fused)
+    e = traced(p, K_HIST, st, [&] { return lbf::launch_hist_update(g, p->bits, d_in, h, nh, st); });
+  return e;
+}
+
 // The fused path on device buffers (a1-a7).  `ws` is the scratch of this call: the FP32
 // corner-turned block, or the FP16 planes of a tensor-core plan (with `maps` their descriptors).
 // input_read (optional) is recorded once d_in has been read; the first kernel that writes d_out
@@ -258,8 +271,6 @@ int bf_kernel_id(lbf_plan_t p) { return p->variant == 1 ? K_BF_FEW : p->variant 
 cudaError_t run_block_device(lbf_plan_t p, const void *d_in, void *d_out, void *ws, const CUtensorMap *maps,
                              cudaStream_t st, cudaEvent_t input_read = nullptr, cudaEvent_t out_free = nullptr) {
   lbf::Geometry g = p->geometry();
-  const void *h = p->hist[p->cur];
-  void *nh = p->hist[p->cur ^ 1];
   if (p->tc) {
     // the filter bank writes the FP16 planes before the delay phase and bandpass; the
     // tensor-core weights carry both (folded tables), the incoherent beam the bandpass
@@ -268,8 +279,7 @@ cudaError_t run_block_device(lbf_plan_t p, const void *d_in, void *d_out, void *
     o.hi = ws;
     o.lo = p->planes > 1 ? static_cast<unsigned char *>(ws) + p->ct16_bytes : nullptr;
     o.kpad = p->kpad;
-    cudaError_t e = traced(p, K_PPF_CT16, st, [&] { return lbf::launch_ppf(g, p->bits, d_in, h, nullptr, nullptr, st, &o); });
-    if (e == cudaSuccess) e = traced(p, K_HIST, st, [&] { return lbf::launch_hist_update(g, p->bits, d_in, h, nh, st); });
+    cudaError_t e = filter_bank(p, K_PPF_CT16, g, d_in, nullptr, nullptr, &o, st);
     if (e == cudaSuccess && input_read) e = cudaEventRecord(input_read, st);
     if (e == cudaSuccess && out_free) e = cudaStreamWaitEvent(st, out_free, 0);
     if (e != cudaSuccess) return e;
@@ -286,8 +296,7 @@ cudaError_t run_block_device(lbf_plan_t p, const void *d_in, void *d_out, void *
   float2 *ct = static_cast<float2 *>(ws);
   g.ppf_stall = p->stall_item;   // failure-detection test hook (one-shot)
   p->stall_item = -1;
-  cudaError_t e = traced(p, K_PPF_CT, st, [&] { return lbf::launch_ppf(g, p->bits, d_in, h, nullptr, ct, st); });
-  if (e == cudaSuccess) e = traced(p, K_HIST, st, [&] { return lbf::launch_hist_update(g, p->bits, d_in, h, nh, st); });
+  cudaError_t e = filter_bank(p, K_PPF_CT, g, d_in, nullptr, ct, nullptr, st);
   if (e == cudaSuccess && input_read) e = cudaEventRecord(input_read, st);
   if (e == cudaSuccess && out_free) e = cudaStreamWaitEvent(st, out_free, 0);
   if (e != cudaSuccess) return e;
@@ -505,10 +514,7 @@ lbf_status lbf_ppf(lbf_plan_t p, const void *d_in, void *d_chan, void *stream) {
   if (!device_ptr(d_in, p->word) || !device_ptr(d_chan, 8)) return LBF_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   const lbf::Geometry g = p->geometry();
-  const void *h = p->hist[p->cur];
-  void *nh = p->hist[p->cur ^ 1];
-  cudaError_t e = traced(p, K_PPF, st, [&] { return lbf::launch_ppf(g, p->bits, d_in, h, (float2 *)d_chan, nullptr, st); });
-  if (e == cudaSuccess) e = traced(p, K_HIST, st, [&] { return lbf::launch_hist_update(g, p->bits, d_in, h, nh, st); });
+  cudaError_t e = filter_bank(p, K_PPF, g, d_in, (float2 *)d_chan, nullptr, nullptr, st);
   if (e != cudaSuccess) return cuda_status(e);
   p->cur ^= 1;
   return LBF_OK;

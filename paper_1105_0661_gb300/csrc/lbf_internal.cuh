@@ -81,7 +81,7 @@ struct PpfGroup {
   int spc;                    // spectra per filter-bank work item (a multiple of 16; both pols)
   int chunks;                 // ceil(M / spc)
   long long first_item;       // first filter-bank work item of this group
-  long long first_hist;       // first history element of this group
+  long long first_stream;     // first (station, subband) stream of this group
   const void *maps;           // device copy of its output's tensor maps (ppf_group_maps), when
                               // the group is in a tensor-store launch class
 };
@@ -91,13 +91,16 @@ struct BfGroup {
   void *out;
   int variant;                // 1 few-beam, 2 many-beam (128-beam tiles), 3 many-beam (64-beam tiles)
   int out_kind;
-  int per_fc;                 // work items per (subband, channel): beam groups or beam tiles
+  int lg;                     // few-beam items: 2^lg channels each (0 for the others)
+  int per_fc;                 // work items per (subband, channel) or 2^lg of them: beam groups or beam tiles
   long long first_item;
 };
 
 // --- launchers (return cudaGetLastError() of the launch) ---
 // a1-a3 (+ a4 when ct or ct16 is given): filter bank; reads history `hist`, block `in`.
-cudaError_t launch_ppf(const Geometry &g, int bits, const void *in, const void *hist,
+// and, where ppf_fuses_history(g) and new_hist is given, writes the next block's history to it
+bool ppf_fuses_history(const Geometry &g);
+cudaError_t launch_ppf(const Geometry &g, int bits, const void *in, const void *hist, void *new_hist,
                        float2 *chan, float2 *ct, cudaStream_t st, const Ct16Out *ct16 = nullptr);
 // batch: persistent grouped filter bank (FP32 corner-turned output), history update, beam former.
 // A grouped launch takes its groups (HOST array, at most kMaxGroups) as a grid-constant kernel
@@ -131,7 +134,7 @@ cudaError_t ppf_group_maps(const PpfGroup &G, void *host_dst);
 cudaError_t launch_ppf_group(int bits, int tc, int tma, const PpfGroup *h_groups, int ngrp, long long total,
                              unsigned long long *counter, int ctas, cudaStream_t st);
 // history update of all groups (DEVICE table: each thread looks up its own element's group)
-cudaError_t launch_hist_group(const PpfGroup *d_groups, int ngrp, long long total, cudaStream_t st);
+cudaError_t launch_hist_group(const PpfGroup *d_groups, int ngrp, long long streams, cudaStream_t st);
 // filter-bank work items (both polarisations of one stream chunk) per (station, subband) stream
 int ppf_items_per_stream(int M, int spc);
 int ppf_ctas_per_sm();
@@ -141,10 +144,11 @@ cudaError_t launch_bf_group(int variant, int out_kind, const BfGroup *h_groups, 
                             unsigned long long *counter, size_t smem, cudaStream_t st);
 int bf_group_residency(int variant, int out_kind, size_t smem);
 int few_beams_per_item();
+int few_log_channels(int M, int S);
 int many_beams_per_item(int variant);   // 128 (variant 2) or 64 (variant 3)
 // AUTO beam-former choice: 1 few-beam, 2 many-beam 128-beam tiles, 3 many-beam 64-beam tiles
 int auto_bf_variant(int B, int S);
-size_t bf_smem_bytes(int variant, int S);
+size_t bf_smem_bytes(int variant, int S, int M);
 // FP32 corner-turned [F][N][S][P][M] -> FP16 [F][N][P][M][kpad] hi/lo planes (split-call TC path)
 cudaError_t launch_ct_to_ct16(const Geometry &g, const float2 *ct, const Ct16Out &o, cudaStream_t st);
 // superstation beam former: sum of delay-compensated stations per group (delay.cu)
@@ -172,8 +176,8 @@ int tc_max_stations();
 int tc_spectra_per_tile();   // TMA box height of the FP16 scratch (spectra per N tile)
 int tc_kpad(int S);
 // history update: new_hist = last H samples of [hist | in]
-cudaError_t launch_hist_update(const Geometry &g, int bits, const void *in, const void *hist,
-                               void *new_hist, cudaStream_t st);
+cudaError_t launch_hist_update(const Geometry &g, int bits, const void *in, const void *hist, void *new_hist,
+                               cudaStream_t st);
 // a4 standalone: chan -> ct
 cudaError_t launch_delay_ct(const Geometry &g, const float2 *chan, float2 *ct, cudaStream_t st);
 // a5-a6 (+ a7): beam former; out_kind selects voltages or fused Stokes; variant 1 few, 2 many

@@ -598,11 +598,24 @@ __device__ __forceinline__ void ppf_item(const Geometry &g, const typename Sampl
   if (kTmaSt && p == 0) bulk_wait_read();   // as above
 }
 
-template <int BITS, int MODE, bool kTma, bool kStall = false>
+// The next block's history of stream sf, samples [e0, e1): the last H samples of [history | block].
+template <typename word>
+__device__ __forceinline__ void copy_history(const Geometry &g, long long sf, int e0, int e1, int tid, int threads,
+                                             const word *__restrict__ in, const word *__restrict__ hist,
+                                             word *__restrict__ nhist) {
+  const word *h = hist + sf * g.H + g.T, *x = in + sf * g.T + (g.T - g.H);
+  word *d = nhist + sf * g.H;
+  const int cut = g.H - g.T;                  // samples before `cut` come from the old history
+#pragma unroll 4
+  for (int e = e0 + tid; e < e1; e += threads) d[e] = e < cut ? h[e] : x[e];
+}
+
+// kHist: the CTA also writes its share of the next block's history (nhist).
+template <int BITS, int MODE, bool kTma, bool kHist, bool kStall = false>
 __global__ void __launch_bounds__(kThreads, 1)
 ppf_kernel(Geometry g, const typename SampleIO<BITS>::word *__restrict__ in,
-           const typename SampleIO<BITS>::word *__restrict__ hist, PpfOut po, int chunks, int spc,
-           const __grid_constant__ PpfMaps maps) {
+           const typename SampleIO<BITS>::word *__restrict__ hist, typename SampleIO<BITS>::word *__restrict__ nhist,
+           PpfOut po, int chunks, int spc, const __grid_constant__ PpfMaps maps) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // The tensor stores read 128-byte-aligned staging buffers: the layout aligns them within itself
   // and the base is declared 128-byte aligned (this kernel has no static shared memory).  Rounding
@@ -614,24 +627,37 @@ ppf_kernel(Geometry g, const typename SampleIO<BITS>::word *__restrict__ in,
   }
   PpfSmem<BITS> &sm = *reinterpret_cast<PpfSmem<BITS> *>(smem_raw);
   int s, f, chunk;
+  auto decode = [&](long long item) {
+    if (MODE == MODE_CT16) {   // stations fastest: neighbouring CTAs fill neighbouring K rows of the
+      s = (int)(item % g.S);   // same (channel) planes
+      const long long rest = item / g.S;
+      chunk = (int)(rest % chunks);
+      f = (int)(rest / chunks);
+    } else {
+      const long long sf = item / chunks;          // stream index s * F + f
+      chunk = (int)(item - sf * chunks);
+      s = (int)(sf / g.F);
+      f = (int)(sf - (long long)s * g.F);
+    }
+  };
   const long long item = blockIdx.x;
-  if (MODE == MODE_CT16) {   // stations fastest: neighbouring CTAs fill neighbouring K rows of the
-    s = (int)(item % g.S);   // same (channel) planes
-    const long long rest = item / g.S;
-    chunk = (int)(rest % chunks);
-    f = (int)(rest / chunks);
-  } else {
-    const long long sf = item / chunks;          // stream index s * F + f
-    chunk = (int)(item - sf * chunks);
-    s = (int)(sf / g.F);
-    f = (int)(sf - (long long)s * g.F);
-  }
+  decode(item);
   ppf_setup(sm.ctl);
   uint32_t ph = 0;
   if (kStall && item == g.ppf_stall)
     ppf_item<BITS, MODE, kTma, true>(g, in, hist, po, s, f, chunk, spc, sm, ph, &maps);
   else
     ppf_item<BITS, MODE, kTma>(g, in, hist, po, s, f, chunk, spc, sm, ph, &maps);
+  // this chunk's share of the next block's history, while the last tiles' tensor stores complete
+  if (kHist) {
+    uint32_t cta, tid;   // read again: kept over the main loop, they cost it registers (spills)
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+    decode(cta);
+    const long long n = g.H;
+    copy_history(g, (long long)s * g.F + f, (int)(n * chunk / chunks), (int)(n * (chunk + 1) / chunks), (int)tid, kThreads,
+                 in, hist, nhist);
+  }
   // the tensor stores of the last tiles complete (read and written) before the CTA's shared
   // memory is released; only thread 0 of each half issued any
   if (kTma && threadIdx.x % kHalf == 0) bulk_wait_all();
@@ -701,50 +727,52 @@ cudaError_t launch_group_t(const PpfTable &T, long long total, unsigned long lon
   return cudaGetLastError();
 }
 
-// History update of every observation of a batch: element i of the concatenated histories.
-__global__ void hist_group_kernel(const PpfGroup *__restrict__ grp, int ngrp, long long total) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    int o = 0;
-    while (o + 1 < ngrp && grp[o + 1].first_hist <= i) ++o;
-    const PpfGroup &G = grp[o];
-    const long long j = i - G.first_hist;
-    const long long sf = j / G.g.H;
-    const int e = (int)(j - sf * G.g.H);
-    const long long src = (long long)G.g.T + e;
-    if (G.bits == 16) {
-      const uint2 *in = (const uint2 *)G.in, *h = (const uint2 *)G.hist;
-      ((uint2 *)G.new_hist)[j] = (src < G.g.H) ? h[sf * G.g.H + src] : in[sf * G.g.T + (src - G.g.H)];
-    } else {
-      const uint32_t *in = (const uint32_t *)G.in, *h = (const uint32_t *)G.hist;
-      ((uint32_t *)G.new_hist)[j] = (src < G.g.H) ? h[sf * G.g.H + src] : in[sf * G.g.T + (src - G.g.H)];
-    }
-  }
+// History update of one observation, one CTA per stream.
+template <typename word>
+__global__ void __launch_bounds__(256)
+hist_update_kernel(Geometry g, const word *__restrict__ in, const word *__restrict__ hist, word *__restrict__ nhist) {
+  copy_history(g, (long long)blockIdx.x, 0, g.H, threadIdx.x, 256, in, hist, nhist);
 }
 
-template <int BITS>
-__global__ void hist_update_kernel(long long total, int H, int T,
-                                   const typename SampleIO<BITS>::word *__restrict__ in,
-                                   const typename SampleIO<BITS>::word *__restrict__ hist,
-                                   typename SampleIO<BITS>::word *__restrict__ nhist) {
-  // new history = samples T .. T+H-1 of [history | block]
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const long long sf = i / H;
-    const int e = (int)(i - sf * H);
-    const long long src = (long long)T + e;
-    nhist[i] = (src < H) ? hist[sf * H + src] : in[sf * T + (src - H)];
+// History update of every observation of a batch: one CTA per stream, whose observation one thread
+// looks up (a search and a division per sample took five times as long).
+__global__ void __launch_bounds__(256) hist_group_kernel(const PpfGroup *__restrict__ grp, int ngrp) {
+  __shared__ int o_s;
+  const long long i = blockIdx.x;
+  if (threadIdx.x == 0) {
+    int lo = 0, hi = ngrp - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (grp[mid].first_stream <= i) lo = mid;
+      else hi = mid - 1;
+    }
+    o_s = lo;
   }
+  __syncthreads();
+  const PpfGroup &G = grp[o_s];
+  const long long sf = i - G.first_stream;
+  const Geometry g = G.g;
+  if (G.bits == 16)
+    copy_history<uint2>(g, sf, 0, g.H, threadIdx.x, 256, (const uint2 *)G.in, (const uint2 *)G.hist, (uint2 *)G.new_hist);
+  else
+    copy_history<uint32_t>(g, sf, 0, g.H, threadIdx.x, 256, (const uint32_t *)G.in, (const uint32_t *)G.hist,
+                           (uint32_t *)G.new_hist);
+}
+
+// spectra per CTA of a plan's own launch (kMinCtas)
+int spectra_per_cta(const Geometry &g) {
+  const long long streams = (long long)g.S * g.F;
+  const long long want = (kMinCtas + streams - 1) / streams;      // chunks per stream wanted
+  return (int)((((long long)g.M + want - 1) / want + kTile - 1) / kTile) * kTile;
 }
 
 template <int BITS, int MODE, bool kTma>
-cudaError_t launch_ppf_t(const Geometry &g, const void *in, const void *hist, PpfOut po, const PpfMaps &maps,
+cudaError_t launch_ppf_t(const Geometry &g, const void *in, const void *hist, void *nhist, PpfOut po, const PpfMaps &maps,
                          cudaStream_t st) {
   using word = typename SampleIO<BITS>::word;
   const long long streams = (long long)g.S * g.F;   // one CTA: both polarisations
   if (streams == 0 || g.M == 0) return cudaSuccess;
-  const long long want = (kMinCtas + streams - 1) / streams;      // chunks per stream wanted
-  const int spc = (int)((((long long)g.M + want - 1) / want + kTile - 1) / kTile) * kTile;
+  const int spc = spectra_per_cta(g);
   const int chunks = (g.M + spc - 1) / spc;
   const long long ctas = streams * chunks;
   if (ctas == 0) return cudaSuccess;
@@ -752,17 +780,18 @@ cudaError_t launch_ppf_t(const Geometry &g, const void *in, const void *hist, Pp
   auto go = [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)ctas, kThreads, smem, st>>>(g, (const word *)in, (const word *)hist, po, chunks, spc, maps);
+    kern<<<(unsigned)ctas, kThreads, smem, st>>>(g, (const word *)in, (const word *)hist, (word *)nhist, po, chunks, spc, maps);
     return cudaGetLastError();
   };
   // the failure-detection test build (FP32 corner turn only) when one CTA is to stall
   if constexpr (MODE == MODE_CT32)
-    if (g.ppf_stall >= 0 && g.ppf_stall < ctas) return go(ppf_kernel<BITS, MODE, kTma, true>);
-  return go(ppf_kernel<BITS, MODE, kTma>);
+    if (g.ppf_stall >= 0 && g.ppf_stall < ctas)
+      return nhist ? go(ppf_kernel<BITS, MODE, kTma, true, true>) : go(ppf_kernel<BITS, MODE, kTma, false, true>);
+  return nhist ? go(ppf_kernel<BITS, MODE, kTma, true>) : go(ppf_kernel<BITS, MODE, kTma, false>);
 }
 
 template <int BITS>
-cudaError_t launch_ppf_bits(const Geometry &g, const void *in, const void *hist, float2 *chan, float2 *ct,
+cudaError_t launch_ppf_bits(const Geometry &g, const void *in, const void *hist, void *nhist, float2 *chan, float2 *ct,
                             const Ct16Out *ct16, cudaStream_t st) {
   PpfOut po{nullptr, nullptr, nullptr, 0};
   PpfMaps maps{};
@@ -776,7 +805,7 @@ cudaError_t launch_ppf_bits(const Geometry &g, const void *in, const void *hist,
     if (e == cudaSuccess && ct16->lo) e = encode_ct16_store_map(&maps.lo, ct16->lo, ct16->kpad, g.M, fc_rows);
     if (e != cudaSuccess) return e;
     maps.has_lo = ct16->lo != nullptr;
-    return launch_ppf_t<BITS, MODE_CT16, true>(g, in, hist, po, maps, st);
+    return launch_ppf_t<BITS, MODE_CT16, true>(g, in, hist, nhist, po, maps, st);
   }
   if (ct) {
     po.f32 = ct;
@@ -784,12 +813,12 @@ cudaError_t launch_ppf_bits(const Geometry &g, const void *in, const void *hist,
     if ((long long)g.S * g.F > 0 && g.M > 0 && g.M % 2 == 0 && (reinterpret_cast<uintptr_t>(ct) & 15) == 0) {
       cudaError_t e = encode_ct32_store_map(&maps.ct, ct, g.S, g.M, (long long)g.F * kN, kCtTma);
       if (e != cudaSuccess) return e;
-      return launch_ppf_t<BITS, MODE_CT32, true>(g, in, hist, po, maps, st);
+      return launch_ppf_t<BITS, MODE_CT32, true>(g, in, hist, nhist, po, maps, st);
     }
-    return launch_ppf_t<BITS, MODE_CT32, false>(g, in, hist, po, maps, st);
+    return launch_ppf_t<BITS, MODE_CT32, false>(g, in, hist, nhist, po, maps, st);
   }
   po.f32 = chan;
-  return launch_ppf_t<BITS, MODE_CHAN, false>(g, in, hist, po, maps, st);
+  return launch_ppf_t<BITS, MODE_CHAN, false>(g, in, hist, nhist, po, maps, st);
 }
 
 }  // namespace
@@ -797,10 +826,10 @@ cudaError_t launch_ppf_bits(const Geometry &g, const void *in, const void *hist,
 int ppf_items_per_stream(int M, int spc) { return (M + spc - 1) / spc; }
 int ppf_ctas_per_sm() { return 1; }
 
-cudaError_t launch_ppf(const Geometry &g, int bits, const void *in, const void *hist, float2 *chan,
+cudaError_t launch_ppf(const Geometry &g, int bits, const void *in, const void *hist, void *new_hist, float2 *chan,
                        float2 *ct, cudaStream_t st, const Ct16Out *ct16) {
-  return bits == 16 ? launch_ppf_bits<16>(g, in, hist, chan, ct, ct16, st)
-                    : launch_ppf_bits<8>(g, in, hist, chan, ct, ct16, st);
+  return bits == 16 ? launch_ppf_bits<16>(g, in, hist, new_hist, chan, ct, ct16, st)
+                    : launch_ppf_bits<8>(g, in, hist, new_hist, chan, ct, ct16, st);
 }
 
 bool ppf_group_tma(const PpfGroup &G) {
@@ -846,27 +875,30 @@ cudaError_t launch_ppf_group(int bits, int tc, int tma, const PpfGroup *h_groups
             : launch_group_t<8, MODE_CT32, false>(T, total, counter, ctas, st);
 }
 
-cudaError_t launch_hist_group(const PpfGroup *d_groups, int ngrp, long long total, cudaStream_t st) {
-  if (total == 0) return cudaSuccess;
-  const long long want = (total + 255) / 256;
-  hist_group_kernel<<<(unsigned)(want < 152LL * 16 ? want : 152LL * 16), 256, 0, st>>>(d_groups, ngrp, total);
+// A block of a few tiles per SM is bound by latency and launches: its filter bank copies the history
+// itself (one subband of 8 stations: 22.5 -> 18.5 us a block).  In larger ones the copy costs the FP32
+// form registers and 2-3 % of its time, more than the kernel of its own (LOFAR block: 13.43 against
+// 12.90 + 0.11 ms; 37 stations, 29 subbands of 255 spectra: 0.607 against 0.579 + 0.019).
+bool ppf_fuses_history(const Geometry &g) {
+  const long long tiles = (long long)g.S * g.F * ((g.M + kTile - 1) / kTile);
+  return tiles > 0 && tiles <= 4 * 152;
+}
+
+cudaError_t launch_hist_update(const Geometry &g, int bits, const void *in, const void *hist, void *new_hist,
+                               cudaStream_t st) {
+  const long long streams = (long long)g.S * g.F;
+  if (streams == 0) return cudaSuccess;
+  if (bits == 16)
+    hist_update_kernel<<<(unsigned)streams, 256, 0, st>>>(g, (const uint2 *)in, (const uint2 *)hist, (uint2 *)new_hist);
+  else
+    hist_update_kernel<<<(unsigned)streams, 256, 0, st>>>(g, (const uint32_t *)in, (const uint32_t *)hist,
+                                                          (uint32_t *)new_hist);
   return cudaGetLastError();
 }
 
-
-cudaError_t launch_hist_update(const Geometry &g, int bits, const void *in, const void *hist,
-                               void *new_hist, cudaStream_t st) {
-  const long long total = (long long)g.S * g.F * g.H;
-  if (total == 0) return cudaSuccess;
-  const int threads = 256;
-  const long long want = (total + threads - 1) / threads;
-  const unsigned blocks = (unsigned)(want < 152LL * 16 ? want : 152LL * 16);
-  if (bits == 16)
-    hist_update_kernel<16><<<blocks, threads, 0, st>>>(total, g.H, g.T, (const uint2 *)in,
-                                                       (const uint2 *)hist, (uint2 *)new_hist);
-  else
-    hist_update_kernel<8><<<blocks, threads, 0, st>>>(total, g.H, g.T, (const uint32_t *)in,
-                                                      (const uint32_t *)hist, (uint32_t *)new_hist);
+cudaError_t launch_hist_group(const PpfGroup *d_groups, int ngrp, long long streams, cudaStream_t st) {
+  if (streams == 0) return cudaSuccess;
+  hist_group_kernel<<<(unsigned)streams, 256, 0, st>>>(d_groups, ngrp);
   return cudaGetLastError();
 }
 

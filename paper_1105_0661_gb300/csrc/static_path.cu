@@ -188,7 +188,7 @@ extern "C" lbf_status lbf_run_block_static(const lbf_config *c, const void *d_in
   if (e == cudaSuccess)
     e = lbf::launch_phase_tables(F, B, S, g.fs, g.f0, g.dtau, reinterpret_cast<int *>(tab + tm.phase0),
                                  reinterpret_cast<float *>(tab + tm.step), st);
-  if (e == cudaSuccess) e = lbf::launch_ppf(g, c->sample_bits, d_in, hist, nullptr, ct, st);
+  if (e == cudaSuccess) e = lbf::launch_ppf(g, c->sample_bits, d_in, hist, nullptr, nullptr, ct, st);
   if (e == cudaSuccess) e = lbf::launch_beamform(g, variant, out_kind, ct, d_out, st);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? LBF_ENOMEM : LBF_ECUDA;
   return LBF_OK;
