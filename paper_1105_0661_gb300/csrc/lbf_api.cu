@@ -71,6 +71,19 @@ cudaError_t encode_ct32_store_map(void *map, void *base, int S, int M, long long
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+cudaError_t encode_chan_store_map(void *map, void *base, int M, long long rows) {
+  PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+  if (!encode) return cudaErrorNotSupported;
+  const cuuint64_t dims[4] = {32, (cuuint64_t)M, (cuuint64_t)kN / 16, (cuuint64_t)rows};
+  const cuuint64_t strides[3] = {(cuuint64_t)kN * 8, 128, (cuuint64_t)M * kN * 8};
+  const cuuint32_t box[4] = {32, 16, (cuuint32_t)kN / 16, 1};
+  const cuuint32_t elem[4] = {1, 1, 1, 1};
+  CUresult r = encode(static_cast<CUtensorMap *>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box,
+                      elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 cudaError_t encode_ct32_tile_map(void *map, const void *base, int rows, int M, long long fc_rows, int nsp) {
   PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
   if (!encode) return cudaErrorNotSupported;

@@ -63,6 +63,9 @@ cudaError_t encode_ct16_store_map(void *map, void *base, int kpad, int M, long l
 // The same for the FP32 corner turn [F*N][S][P][M] float2 (M even): boxes of 16 spectra of one
 // (station, pol) x `nch` consecutive channels.
 cudaError_t encode_ct32_store_map(void *map, void *base, int S, int M, long long fc_rows, int nch);
+// The channelised output [rows = F*S*P][M][N] float2 as 128-byte lines of 16 channels: boxes of 16
+// spectra x the 16 channel blocks of one row, 128-byte swizzle.
+cudaError_t encode_chan_store_map(void *map, void *base, int M, long long rows);
 // ... and as [F*N][rows = S*P][M] float2 for the split beam former's prefetches: boxes of `nsp`
 // spectra of all rows of one channel.
 cudaError_t encode_ct32_tile_map(void *map, const void *base, int rows, int M, long long fc_rows, int nsp);

@@ -25,7 +25,10 @@
 //    thread (m = p & 15, k1 = p >> 4) reads 16 contiguous values, a 16-point DFT over p2 gives
 //    X[k1 + 16 k2]; sixteen lanes then hold sixteen consecutive spectra of one channel (for the
 //    FP32 output the delay phasor and bandpass are applied there).  The output is staged in the
-//    tile's own (by then consumed) FIR buffer in the layout of a tensor-map box -- the FP32
+//    tile's own (by then consumed) FIR buffer in the layout of a tensor-map box -- the channels as
+//    [16 blocks of 16 channels][16 spectra] float2 lines, swizzled (stored from the lanes, 8 bytes to
+//    each of 16 rows per instruction, they took twice as long: 24 stations, 16 subbands 1.02 ms
+//    against 0.53), the FP32
 //    corner turn as [256 channels][16 spectra] float2, the FP16 planes as [256 channels][the
 //    station's two K rows][16 spectra] per plane -- and one thread per half writes it with tensor
 //    stores that drain while the next tile is filtered: written from the lanes, the tile's 64 KB
@@ -117,18 +120,19 @@ struct PpfSmem {
   PpfCtl ctl;
   alignas(16) float4 gain[kN / 2];             // [k1][k2 / 2]: bandpass x delay phasor, pairs of k2
   alignas(16) float2 tw[kN];                   // [k1][p2] = exp(-2 pi i k1 p2 / 256)
-  // per polarisation, two tiles of v_m[p] (132 KB); each tile buffer (258 x 128 bytes) also stages
-  // its tile's output for the tensor stores, so it starts on a 128-byte boundary
-  alignas(128) float2 w[kP][2][kTile][kRowV];
+  // per polarisation, two tiles of v_m[p] (132 KB); each tile buffer also stages its tile's output for
+  // the tensor stores, so it starts on a 1024-byte boundary (the period of their swizzle)
+  struct alignas(1024) Tile { float2 v[kTile][kRowV]; };
+  Tile w[kP][2];
   alignas(16) word in[kStages][kSlot];         // input ring of dual-pol samples (64 KB int16, 32 KB int8)
 };
 static_assert(offsetof(PpfSmem<16>, ctl) == 0 && offsetof(PpfSmem<8>, ctl) == 0, "ring control first");
 static_assert((PpfSmem<16>::kSlot * sizeof(uint2)) % 16 == 0 && (PpfSmem<8>::kSlot * sizeof(uint32_t)) % 16 == 0,
               "ring slots 16-byte aligned");
 static_assert(sizeof(PpfSmem<16>) <= 232448 && sizeof(PpfSmem<8>) <= 232448, "one CTA's shared memory");
-static_assert(offsetof(PpfSmem<16>, w) % 128 == 0 && offsetof(PpfSmem<8>, w) % 128 == 0 &&
-                  (kTile * kRowV * sizeof(float2)) % 128 == 0 && 2 * kN * 64 <= kTile * kRowV * sizeof(float2),
-              "tile buffers 128-byte aligned and large enough to stage both FP16 planes of a tile");
+static_assert(offsetof(PpfSmem<16>, w) % 1024 == 0 && offsetof(PpfSmem<8>, w) % 1024 == 0 &&
+                  2 * kN * 64 <= kTile * kRowV * sizeof(float2),
+              "tile buffers 1024-byte aligned and large enough to stage both FP16 planes of a tile");
 
 // Output modes: the channelised layout, the FP32 corner-turned layout, or the FP16 layout of the
 // tensor-core beam former ([F*N][M/32][Kpad][P][32] with station s in rows k = 2s (re), 2s+1 (im);
@@ -205,7 +209,8 @@ __device__ __forceinline__ void half_sync(uint32_t id) {
 // two K rows of a station x 256 channels (encode_ct16_store_map).
 struct PpfMaps {
   CUtensorMap hi, lo;
-  CUtensorMap ct;   // FP32 corner turn [F*N][S][P][M] float2: boxes of 16 spectra x kCtTma channels
+  CUtensorMap ct;   // FP32 corner turn [F*N][S][P][M] float2: boxes of 16 spectra x kCtTma channels;
+                    // channelised output: boxes of 16 channels x 16 spectra x 16 channel blocks
   int has_lo;
 };
 
@@ -332,7 +337,7 @@ __device__ __forceinline__ void ppf_item(const Geometry &g, const typename Sampl
 
   // this half's two FIR buffers: tile t lives in wbuf[t & 1] (FIR output, transformed in place by
   // pass 1, read by pass 2)
-  float2(*wbuf)[kTile][kRowV] = sm.w[pol];
+  auto *const wbuf = sm.w[pol];
   const uint32_t bar_x = 1 + pol, bar_y = 1 + kP + pol;   // this half's named barriers
   const uint32_t bar_z = 1 + 2 * kP + pol, bar_w = 1 + 3 * kP + pol;   // pass 2 staging (kTmaSt)
   const int m1 = p >> 4, c1 = p & 15;   // pass-1 thread: spectrum m1, column p2 = c1
@@ -366,7 +371,7 @@ __device__ __forceinline__ void ppf_item(const Geometry &g, const typename Sampl
     const int nfr = min(kTile, m_end - mt);
     const long long e0 = (long long)mt * kN - dsh;
     const word *slot = sm.in[t % kStages] + (kDirect ? 0 : (int)(e0 & (kAlign - 1))) + p;
-    float2 *vout = &wbuf[t & 1][0][p];
+    float2 *vout = &wbuf[t & 1].v[0][p];
 #pragma unroll
     for (int q = Q0; q < Q1; ++q) {
       if (kFull || q < nfr)
@@ -397,7 +402,7 @@ __device__ __forceinline__ void ppf_item(const Geometry &g, const typename Sampl
   // ---- FFT pass 1 of tile t, in place: column p2 = c1 of spectrum m1, 16-point DFT over p1,
   // twiddle W256^(p2 k1); the thread reads and writes only its own 16 points
   auto pass1 = [&](int t) {
-    float2 *col = &wbuf[t & 1][m1][c1];
+    float2 *col = &wbuf[t & 1].v[m1][c1];
     float2 a[16];
 #pragma unroll
     for (int p1 = 0; p1 < 16; ++p1) a[p1] = col[16 * p1];
@@ -414,17 +419,33 @@ __device__ __forceinline__ void ppf_item(const Geometry &g, const typename Sampl
     constexpr bool kFullTile = decltype(fullc)::value;
     const int mt = m0 + t * kTile;
     float2 a[16];
-    const float4 *src = reinterpret_cast<const float4 *>(&wbuf[t & 1][m2][16 * k1]);
+    const float4 *src = reinterpret_cast<const float4 *>(&wbuf[t & 1].v[m2][16 * k1]);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const float4 v = src[i];
       a[2 * i] = make_float2(v.x, v.y);
       a[2 * i + 1] = make_float2(v.z, v.w);
     }
-    if constexpr (MODE != MODE_CHAN && kTmaSt) half_sync(bar_z);   // the buffer is read: staging may overwrite it
+    if constexpr (kTmaSt) half_sync(bar_z);   // the buffer is read: staging may overwrite it
     dft16(a);
     const int mg = mt + m2;
     if (MODE == MODE_CHAN) {
+      if constexpr (kTmaSt) {
+        // staging = the tensor store's box [16 channel blocks][16 spectra][16 channels] float2 (128-byte
+        // lines, 16-byte chunks XOR the spectrum mod 8: a half-warp's 16 spectra of one channel meet
+        // banks twice instead of 16 times); spectra past the block's end fall outside the map
+        unsigned char *stg = reinterpret_cast<unsigned char *>(&wbuf[t & 1].v[0][0]);
+        unsigned char *mine = stg + m2 * 128 + (((k1 >> 1) ^ (m2 & 7)) << 4) + (k1 & 1) * 8;
+#pragma unroll
+        for (int k2 = 0; k2 < 16; ++k2) *reinterpret_cast<float2 *>(mine + ((k2 + 8) & 15) * 2048) = a[k2];
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // staging visible to the tensor store
+        half_sync(bar_w);
+        if (p == 0) {
+          tma_store_4d(&maps->ct, smem_u32(stg), 0, mt, 0, (f * g.S + s) * kP + pol);
+          bulk_commit();
+        }
+        return;
+      }
       if (mg < m_end) {
         float2 *dst = po.f32 + ((((long long)f * g.S + s) * kP + pol) * g.M + mg) * kN + k1;
 #pragma unroll
@@ -444,7 +465,7 @@ __device__ __forceinline__ void ppf_item(const Geometry &g, const typename Sampl
           // channel c = k1 + 16 j (j = (k2 + 8) & 15): j >= 16 - kCtTma / 16 goes to the staging
           // box [kCtTma channels][16 spectra] float2, the rest straight to global memory
           constexpr int kJ0 = 16 - kCtTma / 16;
-          unsigned char *stg = reinterpret_cast<unsigned char *>(&wbuf[t & 1][0][0]) + kCtStageOff;
+          unsigned char *stg = reinterpret_cast<unsigned char *>(&wbuf[t & 1].v[0][0]) + kCtStageOff;
           float2 *dst = po.f32 + ((((long long)f * kN + k1) * g.S + s) * kP + pol) * g.M + mg;
           const long long cstep = 16LL * g.S * kP * g.M;
 #pragma unroll
@@ -480,7 +501,7 @@ __device__ __forceinline__ void ppf_item(const Geometry &g, const typename Sampl
         if constexpr (kTmaSt) {
           // staging = the tensor store's box: [256 channels][row 2s, 2s+1][16 spectra] halves per
           // plane (64 bytes per channel), hi plane then lo plane, in this tile's buffer
-          unsigned char *stg = reinterpret_cast<unsigned char *>(&wbuf[t & 1][0][0]);
+          unsigned char *stg = reinterpret_cast<unsigned char *>(&wbuf[t & 1].v[0][0]);
           const int col = odd * 32 + (m2 & ~1) * 2;
 #pragma unroll
           for (int k2 = 0; k2 < 16; ++k2) {
@@ -621,7 +642,7 @@ ppf_kernel(Geometry g, const typename SampleIO<BITS>::word *__restrict__ in,
   // and the base is declared 128-byte aligned (this kernel has no static shared memory).  Rounding
   // the base up at run time instead cost the FP32 form registers (spills); a base that is not
   // aligned after all is reported (device error 5) and the CTA writes nothing.
-  if (kTma && (smem_u32(smem_raw) & 127u) != 0) {
+  if (kTma && (smem_u32(smem_raw) & (MODE == MODE_CHAN ? 1023u : 127u)) != 0) {
     if (threadIdx.x == 0 && g.err) atomicCAS(g.err, 0, DERR_PPF_ALIGN);
     return;
   }
@@ -818,6 +839,12 @@ cudaError_t launch_ppf_bits(const Geometry &g, const void *in, const void *hist,
     return launch_ppf_t<BITS, MODE_CT32, false>(g, in, hist, nhist, po, maps, st);
   }
   po.f32 = chan;
+  const long long rows = (long long)g.S * g.F * kP;
+  if (rows > 0 && rows < (1ll << 31) && g.M > 0 && (reinterpret_cast<uintptr_t>(chan) & 15) == 0) {
+    cudaError_t e = encode_chan_store_map(&maps.ct, chan, g.M, rows);
+    if (e != cudaSuccess) return e;
+    return launch_ppf_t<BITS, MODE_CHAN, true>(g, in, hist, nhist, po, maps, st);
+  }
   return launch_ppf_t<BITS, MODE_CHAN, false>(g, in, hist, nhist, po, maps, st);
 }
 
