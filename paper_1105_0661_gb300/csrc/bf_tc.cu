@@ -32,6 +32,10 @@
 // soon as the MMAs that read the weights they replace are complete: at the item's last tile pair
 // with one weight set (three products), at its first with two (the two-product form).
 //
+// The incoherent beam of a Stokes I plan is summed by two more warps from the stages the MMAs read,
+// which spares the planes a second pass (127 beams of 30 subbands: 1.235 ms for
+// both, 1.227 + 0.928 apart).
+//
 // The epilogue integrates each polarisation component over the window in registers (one shuffle
 // per spectrum for Stokes V) and combines the (Re, Im) row pair with two shuffles per window.
 // Every mbarrier wait is bounded: on expiry the kernel records an error code, stops issuing work,
@@ -59,8 +63,17 @@ constexpr uint32_t kACol0 = kMTiles * kAccCols;   // first weight column (wcol)
 // side of a work item, so more warps per accumulator shorten it.
 template <int NS, int Q>
 __host__ __device__ constexpr int epi_split() { return (NS != 0 && Q <= 16) ? 4 : 2; }
-template <int NS, int Q>
-__host__ __device__ constexpr int tc_threads() { return 64 + 4 * 32 * epi_split<NS, Q>(); }
+// kForm: kMultiPlan (the launch table holds several plans, a batch, each with its own product count)
+// or a single plan -- plan 0, its parameters at compile-time offsets into the table -- with three
+// (kSingle3) or two (kSingle2) products; a run-time product count costs the single plan ~3 %.
+constexpr int kSingle3 = 0, kSingle2 = 1, kMultiPlan = 2;
+// Two more warps of the single-plan Stokes I forms sum the incoherent beam from the same stages.
+template <int NS, int kForm>
+__host__ __device__ constexpr int inc_warps() { return NS == 1 && kForm != kMultiPlan ? 2 : 0; }
+template <int NS, int Q, int kForm>
+__host__ __device__ constexpr int tc_threads() {
+  return 64 + 4 * 32 * epi_split<NS, Q>() + 32 * inc_warps<NS, kForm>();
+}
 
 // One plan of a launch.
 struct TcParams {
@@ -86,6 +99,7 @@ struct TcLaunch {
   TcParams plan[kMaxPlans];
   int nplans, items;          // plans, and work items of all plans
   int nstages, stage_max;     // ring stages, sized for the plan with the largest stage
+  int inc;                    // 1: the incoherent beam too (single-plan Stokes I)
   long long stall_item;       // failure-detection test: the loads stop at this item (-1: never)
 };
 
@@ -388,11 +402,6 @@ __device__ __forceinline__ void flush_stage(const TcParams &p, const float *buf,
   }
 }
 
-// kForm: kMultiPlan (the launch table holds several plans, a batch, each with its own product count)
-// or a single plan -- plan 0, its parameters at compile-time offsets into the table -- with three
-// (kSingle3) or two (kSingle2) products; a run-time product count costs the single plan ~3 %.
-constexpr int kSingle3 = 0, kSingle2 = 1, kMultiPlan = 2;
-
 // TMEM column of the weights of M tile mt: the hi plane (lo = hi + 64 with three products).  The
 // single-plan two-product form needs no lo planes, which leaves room for two weight sets used by
 // alternate items (set = item parity): the next item's weights are written early in the current
@@ -401,8 +410,40 @@ template <int kForm>
 __device__ __forceinline__ uint32_t wcol(int mt, int set) {
   return kForm == kSingle2 ? kACol0 + (uint32_t)(set * 128 + mt * 64) : kACol0 + (uint32_t)(2 * mt * 64);
 }
+// Incoherent beam of one 32-spectrum atom (K rows of 128 bytes at `atom`, hi plane; the lo plane
+// `lo_off` on): lane (pol, j) sums |X|^2 (or |Y|^2) of spectra 2 j, 2 j + 1 over the stations in their
+// order, as incoherent_ct16_kernel does (bit for bit), then the windows of Q spectra meet by shuffles.
+template <int Q>
+__device__ __forceinline__ void incoherent_atom(const unsigned char *atom, uint32_t lo_off, int S, int lane, int m0, int M,
+                                                float b2, float *orow) {
+  const int pol = lane >> 4, j = lane & 15;
+  const uint32_t chunk = (uint32_t)(pol * 4 + (j >> 2)), within = (uint32_t)(j & 3) * 4;
+  auto at = [&](const unsigned char *p) { return __half22float2(*reinterpret_cast<const __half2 *>(p)); };
+  float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int s = 0; s < S; ++s) {
+    const int k = 2 * s;
+    const unsigned char *re = atom + k * 128 + ((chunk ^ (uint32_t)(k & 7)) << 4) + within;
+    const unsigned char *im = atom + (k + 1) * 128 + ((chunk ^ (uint32_t)((k + 1) & 7)) << 4) + within;
+    const float2 xr = __fadd2_rn(at(re), at(re + lo_off)), xi = __fadd2_rn(at(im), at(im + lo_off));
+    acc = __ffma2_rn(xr, xr, __ffma2_rn(xi, xi, acc));
+  }
+  const float ox = __shfl_xor_sync(0xffffffffu, acc.x, 16), oy = __shfl_xor_sync(0xffffffffu, acc.y, 16);
+  const float va = __fmul_rn(b2, acc.x + ox), vb = __fmul_rn(b2, acc.y + oy);
+  const int m = m0 + 2 * j;
+  if (Q == 1) {
+    if (pol == 0 && m < M) orow[m] = va;
+    if (pol == 0 && m + 1 < M) orow[m + 1] = vb;
+  } else {
+    float v = va + vb;
+#pragma unroll
+    for (int o = 1; o < Q / 2; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (pol == 0 && m < M && (2 * j) % Q == 0) orow[m / Q] = v;
+  }
+}
+
 template <int NS, int Q, int kForm>
-__global__ void __launch_bounds__(tc_threads<NS, Q>(), 1)
+__global__ void __launch_bounds__(tc_threads<NS, Q, kForm>(), 1)
 bf_tc_kernel(const __grid_constant__ TcLaunch L) {
   constexpr bool kMulti = kForm == kMultiPlan;
   constexpr int KS = epi_split<NS, Q>();          // epilogue warps per TMEM lane quadrant
@@ -433,7 +474,7 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
   if (tid == 0) {
     for (int s = 0; s < nst; ++s) {
       mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), 1);
+      mbar_init(empty_bar(s), 1 + (inc_warps<NS, kForm>() && L.inc ? 2 : 0));
     }
     for (int mt = 0; mt < kMTiles; ++mt) {
       mbar_init(accf_bar(mt), 1);
@@ -539,6 +580,32 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
         umma_commit(drain_bar);
         volatile int never = 0;
         if (!mbar_wait(drain_bar, 0, &never)) fail(abort_flag, err, ERR_MMA);
+      }
+    }
+  } else if (inc_warps<NS, kForm>() && warp >= 2 + 4 * KS) {
+    // ---------------------------------------------------------------- incoherent beam (one atom per warp)
+    if constexpr (inc_warps<NS, kForm>() != 0) {
+      if (L.inc) {
+        const TcParams &p = L.plan[0];
+        const int a = warp - (2 + 4 * KS);
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < L.items && ok; item += gridDim.x) {
+          const int fc = item / p.items_per_fc;
+          const bool mine = item == fc * p.items_per_fc;   // the first beam block of (f, c)
+          const float bpc = p.bp ? __ldg(&p.bp[fc % kN]) : 1.f;
+          float *const orow = p.out + ((long long)p.B * p.F * kN + fc) * (p.M / Q);
+          for (int t = 0; t < p.ntiles; ++t) {
+            if (!mbar_wait(full_bar(s), ph, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+            if (mine)
+              incoherent_atom<Q>(sbase + kBarBytes + (size_t)s * L.stage_max + (size_t)a * p.Kpad * 128,
+                                 (uint32_t)p.stage_bytes / 2, p.S, lane, (2 * t + a) * kSpec, p.M, bpc * bpc, orow);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty_bar(s));
+            if (++s == nst) { s = 0; ph ^= 1u; }
+          }
+        }
       }
     }
   } else {
@@ -663,7 +730,7 @@ cudaError_t launch_q(TcLaunch &L, int grid, cudaStream_t st) {
   if (smem < kMinSmem) smem = kMinSmem;
   cudaError_t e = cudaFuncSetAttribute(bf_tc_kernel<NS, Q, kForm>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  bf_tc_kernel<NS, Q, kForm><<<grid, tc_threads<NS, Q>(), smem, st>>>(L);
+  bf_tc_kernel<NS, Q, kForm><<<grid, tc_threads<NS, Q, kForm>(), smem, st>>>(L);
   return cudaGetLastError();
 }
 
@@ -747,10 +814,12 @@ int tc_kpad(int S) { return ((2 * S + 15) / 16) * 16; }
 int tc_max_plans_per_launch() { return kMaxPlans; }
 
 cudaError_t launch_bf_tc(const Geometry &g, int out_kind, const void *tm_hi, const void *tm_lo, float *out, int *err,
-                         cudaStream_t st, long long stall_item) {
+                         cudaStream_t st, long long stall_item, bool inc) {
   if (g.M == 0 || g.B == 0) return cudaSuccess;
+  if (inc && out_kind != OUT_STOKES_I) return cudaErrorInvalidValue;
   TcLaunch L;
   L.nplans = 0; L.items = 0; L.nstages = 0; L.stage_max = 0;
+  L.inc = inc ? 1 : 0;
   L.stall_item = stall_item;
   if (!fill_plan(L, 0, g, out_kind, tm_hi, tm_lo, out, err)) return cudaErrorInvalidValue;
   return launch_table(L, out_kind, g.Q, st);
@@ -760,6 +829,7 @@ cudaError_t launch_bf_tc_group(const TcPlanRef *plans, int n, int out_kind, int 
   if (n < 1 || n > kMaxPlans) return cudaErrorInvalidValue;
   TcLaunch L;
   L.nplans = 0; L.items = 0; L.nstages = 0; L.stage_max = 0;
+  L.inc = 0;
   L.stall_item = -1;
   int k = 0;
   for (int i = 0; i < n; ++i) {

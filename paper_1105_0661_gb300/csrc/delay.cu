@@ -117,7 +117,8 @@ incoherent_ct16_kernel(Geometry g, Ct16Out o, float *__restrict__ out) {
     const float b2 = g.ct16_raw ? g.bandpass[c] * g.bandpass[c] : 1.f;
 #pragma unroll
     for (int st = 0; st < NS; ++st) {
-      float v = b2 * (st == 0 ? xx + yy : st == 1 ? xx - yy : st == 2 ? 2.f * re : 2.f * im);
+      // (rounded by itself, as the beam former's own sum of it is)
+      float v = __fmul_rn(b2, st == 0 ? xx + yy : st == 1 ? xx - yy : st == 2 ? 2.f * re : 2.f * im);
       for (int o2 = 1; o2 < g.Q; o2 <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o2);
       if (active && (m & (g.Q - 1)) == 0)
         out[((((long long)g.B * NS + st) * g.F + f) * kN + c) * Mq + m / g.Q] = v;

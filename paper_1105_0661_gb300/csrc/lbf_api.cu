@@ -297,14 +297,15 @@ cudaError_t run_block_device(lbf_plan_t p, const void *d_in, void *d_out, void *
     if (e == cudaSuccess && out_free) e = cudaStreamWaitEvent(st, out_free, 0);
     if (e != cudaSuccess) return e;
     p->cur ^= 1;
-    if (p->inc) {
+    const bool inc = p->inc && p->out_kind == lbf::OUT_STOKES_I;   // summed by the beam former itself
+    if (p->inc && !inc) {
       e = traced(p, K_INC16, st, [&] { return lbf::launch_incoherent_ct16(g, p->out_kind, o, (float *)d_out, st); });
       if (e != cudaSuccess) return e;
     }
     return traced(p, K_BF_TC, st, [&] {
       const long long stall = p->stall_item;
       p->stall_item = -1;
-      return lbf::launch_bf_tc(g, p->out_kind, &maps[0], &maps[1], (float *)d_out, p->d_err, st, stall); });
+      return lbf::launch_bf_tc(g, p->out_kind, &maps[0], &maps[1], (float *)d_out, p->d_err, st, stall, inc); });
   }
   float2 *ct = static_cast<float2 *>(ws);
   g.ppf_stall = p->stall_item;   // failure-detection test hook (one-shot)
@@ -577,13 +578,14 @@ lbf_status lbf_beamform_stokes(lbf_plan_t p, const void *d_ct, float *d_out, voi
     if (p->external_ws) return LBF_EUNSUPPORTED;
     const lbf::Ct16Out o = ct16_out(p);
     cudaError_t e = traced(p, K_CT16, st, [&] { return lbf::launch_ct_to_ct16(g, (const float2 *)d_ct, o, st); });
-    if (e == cudaSuccess && p->inc)
+    const bool inc = p->inc && p->out_kind == lbf::OUT_STOKES_I;
+    if (e == cudaSuccess && p->inc && !inc)
       e = traced(p, K_INC16, st, [&] { return lbf::launch_incoherent_ct16(g, p->out_kind, o, d_out, st); });
     if (e != cudaSuccess) return cuda_status(e);
     return cuda_status(traced(p, K_BF_TC, st, [&] {
       const long long stall = p->stall_item;
       p->stall_item = -1;
-      return lbf::launch_bf_tc(g, p->out_kind, &p->tmap[0], &p->tmap[1], d_out, p->d_err, st, stall); }));
+      return lbf::launch_bf_tc(g, p->out_kind, &p->tmap[0], &p->tmap[1], d_out, p->d_err, st, stall, inc); }));
   }
   return cuda_status(traced(p, bf_kernel_id(p), st, [&] {
     return lbf::launch_beamform(g, p->variant, p->out_kind, (const float2 *)d_ct, d_out, st); }));

@@ -160,9 +160,10 @@ cudaError_t launch_superstation(const Geometry &g, const float2 *ct, float2 *ss,
 // incoherent beam (index B of the Stokes output) from the FP16 planes of a tensor-core plan
 cudaError_t launch_incoherent_ct16(const Geometry &g, int out_kind, const Ct16Out &o, float *out, cudaStream_t st);
 // tcgen05 beam former with fused Stokes epilogue (bf_tc.cu); tm_hi/tm_lo are CUtensorMap*
-// stall_item >= 0: failure-detection test, the loads of that work item are never issued
+// stall_item >= 0: failure-detection test, the loads of that work item are never issued; inc: the
+// incoherent beam too (Stokes I), otherwise launch_incoherent_ct16 forms it
 cudaError_t launch_bf_tc(const Geometry &g, int out_kind, const void *tm_hi, const void *tm_lo, float *out, int *err,
-                         cudaStream_t st, long long stall_item = -1);
+                         cudaStream_t st, long long stall_item = -1, bool inc = false);
 // several tensor-core plans of one output kind and integration length in ONE persistent launch
 // (their work items numbered one after the other); n <= tc_max_plans_per_launch()
 struct TcPlanRef {
