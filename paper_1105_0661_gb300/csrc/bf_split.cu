@@ -141,11 +141,42 @@ __device__ __forceinline__ float2 weight_of(const SpParams &p, int f, int c, int
 constexpr int kEvalWarps = 3;
 constexpr int weight_stage_bytes(int Kpad) { return 3 * (Kpad / 2) * kItemBeams * 4; }
 
-__device__ __forceinline__ void slice_weight(float w, float &w1, float &w2, float &w3) {
-  w1 = fmaf(w, kWUnit, kMagic) - kMagic;
-  const float rest = fmaf(w, kWUnit, -w1);
-  w2 = __half2float(__float2half_rn(rest));
-  w3 = rest - w2;
+// exp(2 pi i phi) of two phases in 2^-32 cycle, as packed operations: reduced to the nearest quarter
+// cycle in integers, then the Taylor polynomials of sine (degree 9) and cosine (degree 10), whose
+// remainders at an eighth of a cycle are 2e-9 and 1e-10 (twice as fast as two general sincos).
+__device__ __forceinline__ void two_phasors(int phi0, int phi1, float2 &w0, float2 &w1) {
+  const int q0 = (int)((unsigned)phi0 + (1u << 29)) >> 30, q1 = (int)((unsigned)phi1 + (1u << 29)) >> 30;
+  const int r0 = (int)((unsigned)phi0 - ((unsigned)q0 << 30)), r1 = (int)((unsigned)phi1 - ((unsigned)q1 << 30));
+  auto both = [](float a) { return make_float2(a, a); };
+  const float2 x = __fmul2_rn(make_float2((float)r0, (float)r1), both(1.4629180792671596e-9f));   // radians
+  const float2 x2 = __fmul2_rn(x, x);
+  float2 s = __ffma2_rn(x2, both(2.7557319e-6f), both(-1.98412698e-4f));
+  s = __ffma2_rn(x2, s, both(8.3333333e-3f));
+  s = __ffma2_rn(x2, s, both(-1.66666667e-1f));
+  s = __ffma2_rn(__fmul2_rn(x2, s), x, x);
+  float2 c = __ffma2_rn(x2, both(-2.7557319e-7f), both(2.48015873e-5f));
+  c = __ffma2_rn(x2, c, both(-1.38888889e-3f));
+  c = __ffma2_rn(x2, c, both(4.16666667e-2f));
+  c = __ffma2_rn(x2, c, both(-0.5f));
+  c = __ffma2_rn(x2, c, both(1.f));
+  auto turn = [](int q, float s, float c) {
+    const float a = (q & 1) ? -s : c, b = (q & 1) ? c : s;
+    return (q & 2) ? make_float2(-a, -b) : make_float2(a, b);
+  };
+  w0 = turn(q0, s.x, c.x);
+  w1 = turn(q1, s.y, c.y);
+}
+
+// slices of (cos, sin), each a half2
+__device__ __forceinline__ void slice_weight(float2 w, uint32_t &w1, uint32_t &w2, uint32_t &w3) {
+  const float2 u = make_float2(kWUnit, kWUnit), mg = make_float2(kMagic, kMagic), m1 = make_float2(-1.f, -1.f);
+  const float2 h = __ffma2_rn(__ffma2_rn(w, u, mg), m1, mg);    // minus the integer part
+  const float2 rest = __ffma2_rn(w, u, h);
+  const __half2 second = __floats2half2_rn(rest.x, rest.y);
+  const float2 third = __ffma2_rn(__half22float2(second), m1, rest);
+  w1 = pack_half2(-h.x, -h.y);
+  w2 = *reinterpret_cast<const uint32_t *>(&second);
+  w3 = pack_half2(third.x, third.y);
 }
 
 // Beams fastest over the lanes of a warp, so that the stage is written without bank conflicts; a
@@ -158,18 +189,21 @@ __device__ __forceinline__ void eval_weights(const SpParams &p, uint32_t *stage,
     const int s0 = (u >> 1) * 4, bl = (u & 1) * 32 + lane, b = it.bb * kItemBeams + bl;
     const int *ph = p.phase0 + ((long long)f * p.B + b) * p.S;
     const float *st = p.step + (long long)b * p.S;
+    int phi[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int s = s0 + k;
-      float2 w = make_float2(0.f, 0.f);
-      if (b < p.B && s < p.S) w = fixed_phasor(weight_phase(__ldg(ph + s), __ldg(st + s), dc));
-      float x1, x2, x3, y1, y2, y3;
-      slice_weight(w.x, x1, x2, x3);
-      slice_weight(w.y, y1, y2, y3);
-      uint32_t *d = stage + s * kItemBeams + bl;
-      d[0] = pack_half2(x1, y1);
-      d[S2 * kItemBeams] = pack_half2(x2, y2);
-      d[2 * S2 * kItemBeams] = pack_half2(x3, y3);
+    for (int k = 0; k < 4; ++k)
+      phi[k] = b < p.B && s0 + k < p.S ? weight_phase(__ldg(ph + s0 + k), __ldg(st + s0 + k), dc) : 0;
+#pragma unroll
+    for (int k = 0; k < 4; k += 2) {
+      float2 w[2];
+      two_phasors(phi[k], phi[k + 1], w[0], w[1]);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int s = s0 + k + e;
+        if (b >= p.B || s >= p.S) w[e] = make_float2(0.f, 0.f);
+        uint32_t *d = stage + s * kItemBeams + bl;
+        slice_weight(w[e], d[0], d[S2 * kItemBeams], d[2 * S2 * kItemBeams]);
+      }
     }
   }
 }
@@ -524,12 +558,12 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
     const bool inf = group_sync_any(1 + grp, 32 * kGroup,
                                     fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) > 3.402823466e38f);
     if (gfail[grp * 2 + (n & 1)]) break;      // the whole group leaves together
-    // scale 2^(137 - E) for a peak in [2^(E - 127), 2^(E - 126)): the peak lands in [2^10, 2^11);
-    // its inverse, with the weights' 2^7, is 2^(E - 144) (subnormal for E < 18)
+    // scale 2^(137 - E) for a peak in [2^(E - 127), 2^(E - 126)), E >= 10: the peak lands in
+    // [2^10, 2^11); its inverse, with the weights' 2^7, is 2^(E - 127) 2^-17
     auto scale_of = [](uint32_t cb, float &inv) {
-      const int E = max((int)(cb >> 23), 10);
-      inv = E >= 18 ? __uint_as_float((uint32_t)(E - 17) << 23) : __uint_as_float(1u << (E + 5));
-      return __uint_as_float((uint32_t)(264 - min(E, 254)) << 23);
+      const uint32_t e = max(cb & 0x7f800000u, 10u << 23);
+      inv = __uint_as_float(e) * 7.62939453125e-6f;
+      return __uint_as_float((264u << 23) - e);
     };
     float4 inv;
     const float sc[4] = {scale_of(cm[0], inv.x), scale_of(cm[16], inv.y), scale_of(cm[32], inv.z),
@@ -539,7 +573,7 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
     // station s0 + 8 i holds rows k = 2 s0 + 16 i (re) and k + 1 (im).  (After an expired wait the
     // stage is overwritten all the same: the launch has failed.)
     const uint32_t chunk = (uint32_t)(pol * 4 + (j >> 1)), within = (uint32_t)(j & 1) * 8;
-    const int k0 = 2 * s0;
+    const int k0 = 2 * s0, steps = Kpad / (4 * kGroup);
     unsigned char *re = sbase + kRingOff + (size_t)s * L.stage_max + (size_t)grp * (Kpad * 128) + k0 * 128 + within;
     unsigned char *im = re + 128 + ((chunk ^ (uint32_t)((k0 + 1) & 7)) << 4);
     re += (chunk ^ (uint32_t)(k0 & 7)) << 4;
@@ -562,7 +596,7 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
         h[e] = __ffma2_rn(__ffma2_rn(x, sx, mg), m1, mg);   // minus the leading slice
         l[e] = __ffma2_rn(x, sx, h[e]);
       }
-      if (k0 + 4 * kGroup * i < Kpad) {
+      if (i < steps) {
         *reinterpret_cast<uint2 *>(re + i * (kGroup * 512)) = make_uint2(pack_half2(-h[0].x, -h[1].x), pack_half2(-h[2].x, -h[3].x));
         *reinterpret_cast<uint2 *>(im + i * (kGroup * 512)) = make_uint2(pack_half2(-h[0].y, -h[1].y), pack_half2(-h[2].y, -h[3].y));
         *reinterpret_cast<uint2 *>(re + lo_off + i * (kGroup * 512)) = make_uint2(pack_half2(l[0].x, l[1].x), pack_half2(l[2].x, l[3].x));
