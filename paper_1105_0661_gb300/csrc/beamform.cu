@@ -84,6 +84,7 @@ __device__ __forceinline__ void bf_few_item(const Geometry &g, const float2 *__r
     const int s = i / FB, b = b0 + (i - s * FB);
     wsm[i] = (b < g.B) ? beam_weight(g, f, c, (long long)b * g.S + s) : make_float2(0.f, 0.f);
   }
+  wait_for_previous();
   __syncthreads();
   const float2 *y = ct + (long long)fc * g.S * kP * g.M;
   const int nS = (OUT == OUT_STOKES_IQUV) ? 4 : 1;
@@ -180,8 +181,7 @@ cudaError_t launch_few(const Geometry &g, int out_kind, const float2 *ct, void *
   auto go = [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kFewThreads, smem, st>>>(g, ct, out, lg);
-    return cudaGetLastError();
+    return launch_behind(g.pdl != 0, kern, grid, kFewThreads, smem, st, g, ct, out, lg);
   };
   switch (out_kind) {
     case OUT_VOLTAGES: return lg ? go(bf_few_kernel<OUT_VOLTAGES, 8, false>) : go(bf_few_kernel<OUT_VOLTAGES, 8, true>);

@@ -38,6 +38,7 @@ struct Geometry {
   int ct16_raw = 0;           // 1: the FP16 planes hold the filtered spectrum before the delay phase
                               // and bandpass, which the tensor-core weights then carry
   int *err = nullptr;                   // device error word: a bounded wait that gave up records here
+  int pdl = 0;                          // 1: launch behind the previous kernel's tail (launch_behind)
   long long ppf_stall = -1;             // failure-detection test: this filter-bank CTA issues no input copies
 };
 
@@ -214,7 +215,30 @@ int many_beam_max_stations();
 cudaError_t launch_stokes(const Geometry &g, int out_kind, const float2 *vol, float *out,
                           cudaStream_t st);
 
+// Launch `kern`; with `pdl` as a programmatic dependent launch: its CTAs may start while the kernel
+// before it on the stream still runs (once that has called let_dependents_start in every CTA, or has
+// ended), and must call wait_for_previous before they read or write what it writes or reads.  Saves a
+// small block most of a launch's latency.
+template <typename... P, typename... A>
+cudaError_t launch_behind(bool pdl, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // Shared device helpers --------------------------------------------------------------------------
+// Programmatic dependent launch (launch_behind); both do nothing in an ordinary launch.
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_dependents_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }

@@ -664,6 +664,8 @@ ppf_kernel(Geometry g, const typename SampleIO<BITS>::word *__restrict__ in,
   const long long item = blockIdx.x;
   decode(item);
   ppf_setup(sm.ctl);
+  let_dependents_start();
+  wait_for_previous();
   uint32_t ph = 0;
   if (kStall && item == g.ppf_stall)
     ppf_item<BITS, MODE, kTma, true>(g, in, hist, po, s, f, chunk, spc, sm, ph, &maps);
@@ -801,8 +803,8 @@ cudaError_t launch_ppf_t(const Geometry &g, const void *in, const void *hist, vo
   auto go = [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)ctas, kThreads, smem, st>>>(g, (const word *)in, (const word *)hist, (word *)nhist, po, chunks, spc, maps);
-    return cudaGetLastError();
+    return launch_behind(g.pdl != 0, kern, dim3((unsigned)ctas), kThreads, smem, st, g, (const word *)in, (const word *)hist,
+                         (word *)nhist, po, chunks, spc, maps);
   };
   // the failure-detection test build (FP32 corner turn only) when one CTA is to stall
   if constexpr (MODE == MODE_CT32)
