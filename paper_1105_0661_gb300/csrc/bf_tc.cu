@@ -60,9 +60,14 @@ constexpr uint32_t kACol0 = kMTiles * kAccCols;   // first weight column (wcol)
 
 // Epilogue warps per TMEM lane quadrant: 4 for Stokes outputs whose windows fit in 16 spectra (each
 // warp drains 16 spectra of an accumulator), else 2 (32 spectra each).  The epilogue is the longer
-// side of a work item, so more warps per accumulator shorten it.
+// side of a work item, so more warps per accumulator shorten it.  IQUV in windows of one or two
+// spectra is bound by its output rows instead, which two warps write in runs twice as long (16
+// subbands, 127 beams, 768 spectra: Q = 1 2.52 -> 1.80 ms, Q = 2 1.68 -> 1.20; Stokes I at Q = 1 went
+// from 0.88 to 1.23 that way and keeps four).
 template <int NS, int Q>
-__host__ __device__ constexpr int epi_split() { return (NS != 0 && Q <= 16) ? 4 : 2; }
+__host__ __device__ constexpr int epi_split() {
+  return (NS == 1 && Q <= 16) || (NS == 4 && Q >= 4 && Q <= 16) ? 4 : 2;
+}
 // kForm: kMultiPlan (the launch table holds several plans, a batch, each with its own product count)
 // or a single plan -- plan 0, its parameters at compile-time offsets into the table -- with three
 // (kSingle3) or two (kSingle2) products; a run-time product count costs the single plan ~3 %.
@@ -187,7 +192,7 @@ constexpr int kVStageBytes = 8 * 2 * kSpec * 8;   // voltages: 8 beams x 2 pols 
 // kWin windows, the 16-byte chunks of a beam XOR-swizzled by the beam index; two buffers alternate.
 // Shorter windows go through each warp's short rows (tc_ptx.cuh).  Measured, 300 beams IQUV over 4 of
 // 40 stations, 24 subbands of 384 spectra (2.8 GB of output): 9.73 ms with the
-// scattered stores, 1.94 staged; 128 beams IQUV unintegrated: 32.1 and 1.87.
+// scattered stores, 1.94 staged; 128 beams IQUV unintegrated: 32.1 and 1.87 (runs of 16, see epi_split).
 template <int NS, int Q>
 struct Stage {
   static constexpr bool kOn = NS != 0 && Q >= 4;
@@ -196,7 +201,7 @@ struct Stage {
   static constexpr int kParts = kWin / 4;                      // 16-byte parts of a row segment
   static constexpr int kRow = NS * kWin;                       // floats per beam (0: voltages)
   static constexpr int kBuf = 32 * kRow;                       // floats per quadrant buffer
-  using Rows = ShortRows<NS == 0 ? 1 : NS, Q <= 2 ? 16 / Q : 8>;
+  using Rows = ShortRows<NS == 0 ? 1 : NS, Q <= 2 ? 2 * kSpec / epi_split<NS, Q>() / Q : 8>;   // a drained tile's windows
   static constexpr int kBytes = NS == 0 ? 8 * kVStageBytes       // voltages: 4 KB per epilogue warp
                                         : kOn ? 4 * 2 * kBuf * 4   // 4 quadrants x 2 buffers
                                               : 4 * epi_split<NS, Q>() * Rows::kBytes;
