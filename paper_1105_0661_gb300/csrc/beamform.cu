@@ -486,9 +486,14 @@ cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct,
 // stations 24 beams 0.29 / 0.30, 24 stations 12 beams 0.32 / 0.33, 48 stations 9 beams 0.58 / 0.37.
 // A handful of stations over a tile of spectra is all weights: 4 stations, 64 beams, 64 spectra of 16
 // subbands 0.060 / 0.066 (many-beam kernel / split), 4 stations, 40 beams, 768 spectra 0.16 / 0.10.
+// The incoherent beam costs the split kernel a pass of its own over the block, which the few-beam
+// kernel's one pass for up to 16 beams of Stokes I saves: 16 subbands, few-beam / split and the pass:
+// 12 beams of 16 stations 0.437 / 0.475 ms, of 64 1.20 / 1.26; 16 beams of 64 stations 1.25 / 1.28;
+// 24 beams of 16 stations 0.68 / 0.48.
 bool beamform_uses_split(const Geometry &g, int variant, int out_kind) {
   if (g.S > split_max_stations()) return false;
   if (variant != 1) return g.S >= 8 || g.M >= 256;
+  if (g.inc && out_kind == OUT_STOKES_I && g.B <= 16) return false;
   return g.B > 8 && (g.B + 7) / 8 * g.S >= (out_kind == OUT_VOLTAGES ? 56 : 24);
 }
 
@@ -592,7 +597,8 @@ size_t bf_smem_bytes(int variant, int S, int M) {
   return (size_t)S * ((variant == 3 ? 64 : kBT) + 2 * kP * kMC) * sizeof(float2);
 }
 
-// Beam-former choice for AUTO: the few-beam kernel up to 32 beams (it reads the block once per 8
+// Beam-former choice for AUTO where the split kernel does not serve the plan (beamform_uses_split):
+// the few-beam kernel up to 32 beams (it reads the block once per 8
 // beams at HBM speed; a 64-beam FP32 tile costs about as much as 6 such passes); beyond, the
 // many-beam tile (128 or 64 beams per CTA) that leaves the fewest tile slots empty, a 64-beam slot
 // counted as 1.15 of a 128-beam one (the narrower tile issues more shared loads per FMA).
