@@ -6,8 +6,9 @@
 // same registers and shared memory, so that each body runs as it does alone: the filter bank per
 // (sample width, FP32 or FP16-plane output, tensor-store output or not -- each observation's
 // tensor maps sit in a device array its table entry points at), one history launch, the FP32 beam former per
-// (kernel variant, output kind, CTAs per SM), and one tensor-core launch per (output kind,
-// integration length), whose work items number the class's plans one after the other.
+// (kernel variant, output kind, CTAs per SM) or, where the split kernel serves a plan, per (output
+// kind, integration length), and one tensor-core launch per (output kind, integration length); the
+// work items of these two number the class's plans one after the other.
 //
 // A batch can be captured as CUDA graphs (one per history parity: each block flips every plan's
 // history ping-pong) and replayed with a single graph launch per block.  Its shapes -- spectra per

@@ -42,10 +42,10 @@
 //  * epilogue warps (8): warp w serves TMEM lane quadrant w % 4 and one 32-spectrum half.  They take
 //    D2 into registers while the MMAs fill D1, and D1 while the MMAs fill the next tile's D2, so
 //    that one accumulator of each suffices (256 TMEM columns, next to 4 x 64 of weight slices).
-// What bounds it: the issue slots (ncu, 8 subbands of the LOFAR block: 61 % of them used, 7900 warp
+// What bounds it: the issue slots (ncu, 8 subbands of the LOFAR block: 61 % of them used, 7400 warp
 // instructions per tile of 64 beams, half of them the converters', a quarter the epilogue's) and the
 // latency of the converters' chain; the MMAs take half of a tile's 3300 cycles.  127 beams of the
-// LOFAR block: 86.2 ms in FP32 FMAs, 17.0 here; 37 beams of 30 subbands: 5.5 ms and 1.07; voltages of
+// LOFAR block: 86.2 ms in FP32 FMAs, 16.5 here; 37 beams of 30 subbands: 5.5 ms and 1.07; voltages of
 // 127 beams, 16 subbands: 5.7 ms and 1.8.
 // Every mbarrier wait is bounded: on expiry the kernel records an error code, stops issuing work,
 // waits (bounded) for its MMAs in flight, frees TMEM and returns.  The MMA thread, the evaluators and
@@ -62,7 +62,7 @@ constexpr int kItemBeams = kRows / 2;       // 64 beams per work item
 constexpr int kTileSpec = 2 * kSpec;        // 64 spectra per tile
 constexpr int kEpiWarps = 8, kConvWarps = 8;
 constexpr int kGroup = kConvWarps / 2;      // converter warps per half tile
-constexpr int kThreads = 128 + 32 * (kEpiWarps + kConvWarps);   // warpgroup 0: MMA issuer (and 3 idle warps)
+constexpr int kThreads = 128 + 32 * (kEpiWarps + kConvWarps);   // warpgroup 0: MMA issuer and 3 weight evaluators
 constexpr int kMaxStages = 4;
 constexpr int kBarBytes = 1024;
 constexpr int kSlots = 8;                   // column-scale ring: more than the stages + 3 tiles in flight

@@ -191,7 +191,7 @@ class Dims:
 class Plan:
     """One observation: tables, device-resident FIR/shift history and run_block scratch.
 
-    precision: "fp32" (SIMT), "fp16tc" (tensor cores, three FP16 products) or "fp16tc2" (tensor
+    precision: "fp32" (errors of FP32 arithmetic), "fp16tc" (tensor cores, three FP16 products) or "fp16tc2" (tensor
     cores, two products: FP16 weights); bf_variant: "auto", "few", "many" (128-beam tiles) or
     "many64" (lbf_config's fields of the same names)."""
 
