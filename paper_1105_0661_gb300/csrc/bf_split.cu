@@ -42,7 +42,7 @@
 //  * epilogue warps (8): warp w serves TMEM lane quadrant w % 4 and one 32-spectrum half.  They take
 //    D2 into registers while the MMAs fill D1, and D1 while the MMAs fill the next tile's D2, so
 //    that one accumulator of each suffices (256 TMEM columns, next to 4 x 64 of weight slices).
-// What bounds it: the issue slots (ncu, 8 subbands of the LOFAR block: 61 % of them used, 7400 warp
+// What bounds it: the issue slots (ncu, 8 subbands of the LOFAR block: 57 % of them used, 7300 warp
 // instructions per tile of 64 beams, half of them the converters', a quarter the epilogue's) and the
 // latency of the converters' chain; the MMAs take half of a tile's 3300 cycles.  127 beams of the
 // LOFAR block: 86.2 ms in FP32 FMAs, 16.5 here; 37 beams of 30 subbands: 5.5 ms and 1.07; voltages of
