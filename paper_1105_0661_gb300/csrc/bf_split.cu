@@ -281,11 +281,10 @@ __device__ __forceinline__ void flush_stage(const SpParams &p, const float *buf,
   }
 }
 
-// Windows per flush of the short rows: one or both 16-spectrum chunks of a half tile (16, 16, 8).
+// Windows of a half tile for the short rows (Q 2 and 4).
 template <int Q>
 struct Short {
-  static constexpr int kFlushCh = Q == 1 ? 1 : 2;
-  static constexpr int kW = 16 * kFlushCh / Q;
+  static constexpr int kW = Q <= 4 ? kSpec / Q : 8;
 };
 
 // Stokes parameters of one 32-spectrum half tile (spectra m0 .. m0 + 31) from this lane's voltage
@@ -299,6 +298,54 @@ __device__ __forceinline__ void stokes_half(const float2 (&vx)[16], const float2
   constexpr int kW = Q >= 16 ? 1 : 16 / Q;     // windows that end in 16 spectra
   const int ro = lane & 1, jq = lane >> 1;
   const int Mq = M / Q;
+  if constexpr (Q == 1) {
+    // Every spectrum is a window: the parameters replace the voltages, and a whole half tile leaves as
+    // 128-byte rows, the second parameter of each lane after the first (Stokes I, 40 beams of 2
+    // stations, 4 subbands of 768 spectra: 316 us through 16-window short rows, 131 here).
+    float p0[kSpec], p1[kSpec];
+#pragma unroll
+    for (int i = 0; i < kSpec; ++i) {
+      const float x = i & 1 ? vx[i >> 1].y : vx[i >> 1].x, y = i & 1 ? vy[i >> 1].y : vy[i >> 1].x;
+      if (NS == 1) {
+        const float own = x * x + y * y;
+        p0[i] = own + __shfl_xor_sync(0xffffffffu, own, 1);
+      } else {
+        const float yp = __shfl_xor_sync(0xffffffffu, y, 1);   // the partner lane's Y component
+        const float xx = x * x, yy = y * y, v = x * yp;
+        const float i_own = xx + yy, q_own = xx - yy, u_own = x * y, v_own = ro ? v : -v;
+        float k0 = ro ? u_own : i_own, k1 = ro ? v_own : q_own;
+        k0 += __shfl_xor_sync(0xffffffffu, ro ? i_own : u_own, 1);
+        k1 += __shfl_xor_sync(0xffffffffu, ro ? q_own : v_own, 1);
+        p0[i] = ro ? 2.f * k0 : k0;
+        p1[i] = ro ? 2.f * k1 : k1;
+      }
+    }
+#pragma unroll
+    for (int pass = 0; pass < (NS == 4 ? 2 : 1); ++pass) {
+      if (NS == 1) {
+#pragma unroll
+        for (int i = 0; i < kSpec / 2; ++i) wstage[jq * kSpec + ((2 * i + ro) ^ (2 * jq))] = ro ? p0[2 * i + 1] : p0[2 * i];
+      } else {
+#pragma unroll
+        for (int i = 0; i < kSpec; ++i) wstage[lane * kSpec + (i ^ lane)] = pass ? p1[i] : p0[i];
+      }
+      __syncwarp();
+      float *dst = row0 + pass * pstride + m0 + lane;
+      const int nb = m0 + lane < M ? nbeams : 0;
+#pragma unroll 8
+      for (int b = 0; b < 16; ++b, dst += bstride)
+        if (b < nb) {
+          if (NS == 1) {
+            dst[0] = wstage[b * kSpec + (lane ^ (2 * b))];
+          } else {
+            dst[0] = wstage[2 * b * kSpec + (lane ^ (2 * b))];
+            dst[2 * pstride] = wstage[(2 * b + 1) * kSpec + (lane ^ (2 * b + 1))];
+          }
+        }
+      __syncwarp();   // the rows are rewritten by the next pass
+    }
+    return;
+  }
   float2 pxx = make_float2(0.f, 0.f), pyy = pxx, pxy = pxx, pv = pxx;
 #pragma unroll
   for (int ch = 0; ch < 2; ++ch) {
@@ -328,7 +375,7 @@ __device__ __forceinline__ void stokes_half(const float2 (&vx)[16], const float2
           }
         }
       } else {
-        ShortRows<NS, Short<Q>::kW>::put(wstage, lane, Short<Q>::kFlushCh == 2 ? ch * kW + w : w, r0, r1);
+        ShortRows<NS, Short<Q>::kW>::put(wstage, lane, ch * kW + w, r0, r1);
       }
     };
 #pragma unroll
@@ -336,10 +383,7 @@ __device__ __forceinline__ void stokes_half(const float2 (&vx)[16], const float2
       const float2 x = vx[ch * 8 + i], y = vy[ch * 8 + i];
       float2 yp = make_float2(0.f, 0.f);       // the partner lane's Y component
       if (NS == 4) yp = make_float2(__shfl_xor_sync(0xffffffffu, y.x, 1), __shfl_xor_sync(0xffffffffu, y.y, 1));
-      if constexpr (Q == 1) {
-        finish(2 * i, x.x * x.x, y.x * y.x, x.x * y.x, x.x * yp.x);
-        finish(2 * i + 1, x.y * x.y, y.y * y.y, x.y * y.y, x.y * yp.y);
-      } else {
+      {
         pxx = __ffma2_rn(x, x, pxx);
         pyy = __ffma2_rn(y, y, pyy);
         if (NS == 4) {
@@ -353,9 +397,7 @@ __device__ __forceinline__ void stokes_half(const float2 (&vx)[16], const float2
       }
     }
     if constexpr (!Stage<NS, Q>::kOn)
-      if (Short<Q>::kFlushCh == 1 || ch == 1)
-        ShortRows<NS, Short<Q>::kW>::flush(wstage, lane, nbeams, Short<Q>::kFlushCh == 1 ? w0 : m0 / Q, Mq, row0, bstride,
-                                           pstride);
+      if (ch == 1) ShortRows<NS, Short<Q>::kW>::flush(wstage, lane, nbeams, m0 / Q, Mq, row0, bstride, pstride);
   }
 }
 
