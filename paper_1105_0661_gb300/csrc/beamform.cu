@@ -484,17 +484,38 @@ cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct,
 // few-beam / split: Stokes I, 16 subbands: 8 stations 16 beams 0.33 / 0.33 ms, 12 stations 16 beams
 // 0.40 / 0.35, 48 stations 16 beams 0.99 / 0.53 and 8 beams 0.51 / 0.51; voltages, 8 subbands: 12
 // stations 24 beams 0.29 / 0.30, 24 stations 12 beams 0.32 / 0.33, 48 stations 9 beams 0.58 / 0.37.
-// A handful of stations over a tile of spectra is all weights: 4 stations, 64 beams, 64 spectra of 16
-// subbands 0.060 / 0.066 (many-beam kernel / split), 4 stations, 40 beams, 768 spectra 0.16 / 0.10.
+// With a handful of stations the split kernel's weights (short blocks) and its epilogue (unintegrated
+// output, where the FMA kernels are bound by the output alone) weigh most; where the line lies, 4
+// subbands, 40 beams, many-beam kernel / split in us: Stokes I 768 spectra Q = 1, 4 stations 104 / 131,
+// 8 stations 162 / 132; 64 spectra, 12 stations 31 / 31; IQUV Q = 1, 768 spectra, 12 stations 268 / 300,
+// 16 stations 330 / 305, 128 spectra, 16 stations 51 / 54; voltages 768 spectra, 6 stations 144 / 154.
 // The incoherent beam costs the split kernel a pass of its own over the block, which the few-beam
 // kernel's one pass for up to 16 beams of Stokes I saves: 16 subbands, few-beam / split and the pass:
 // 12 beams of 16 stations 0.437 / 0.475 ms, of 64 1.20 / 1.26; 16 beams of 64 stations 1.25 / 1.28;
 // 24 beams of 16 stations 0.68 / 0.48.
+static int split_min_stations(const Geometry &g, int out_kind) {
+  const bool brief = g.M < 256;
+  if (out_kind == OUT_STOKES_IQUV && g.Q == 1) return brief ? 24 : 16;
+  if (out_kind == OUT_VOLTAGES || (out_kind == OUT_STOKES_I && g.Q <= 2)) return brief ? 16 : 8;
+  return g.M < 512 ? 8 : out_kind == OUT_STOKES_I && g.Q <= 4 ? 4 : 1;
+}
+
+// Passes of the few-beam kernel times stations from which the split kernel takes its beams: short
+// windows raise the split kernel's epilogue.  4 subbands of 768 spectra, few-beam / split as a ratio:
+// Stokes I Q = 4: 16 stations 2 passes 0.83, 12 stations 3 passes over 1; Q = 2: 32 stations 2 passes
+// 0.90, 24 stations 3 passes over 1; Q = 1: 24 stations 2 passes 0.97, 32 over 1; IQUV Q = 1: 24
+// stations 2 passes 0.85, 32 over 1, Q >= 2: over 1 from 24.
+static int split_min_passes(const Geometry &g, int out_kind) {
+  if (out_kind == OUT_VOLTAGES || g.Q == 1) return 56;
+  if (out_kind == OUT_STOKES_IQUV) return 24;
+  return g.Q == 2 ? 72 : g.Q <= 8 ? 36 : 24;
+}
+
 bool beamform_uses_split(const Geometry &g, int variant, int out_kind) {
-  if (g.S > split_max_stations()) return false;
-  if (variant != 1) return g.S >= 8 || g.M >= 256;
+  if (g.S > split_max_stations() || g.S < split_min_stations(g, out_kind)) return false;
+  if (variant != 1) return true;
   if (g.inc && out_kind == OUT_STOKES_I && g.B <= 16) return false;
-  return g.B > 8 && (g.B + 7) / 8 * g.S >= (out_kind == OUT_VOLTAGES ? 56 : 24);
+  return g.B > 8 && (g.B + 7) / 8 * g.S >= split_min_passes(g, out_kind);
 }
 
 cudaError_t launch_beamform(const Geometry &g, int variant, int out_kind, const float2 *ct, void *out,
