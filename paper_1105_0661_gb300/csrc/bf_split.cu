@@ -610,7 +610,7 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
     float4 inv;
     const float sc[4] = {scale_of(cm[0], inv.x), scale_of(cm[16], inv.y), scale_of(cm[32], inv.z),
                          scale_of(cm[48], inv.w)};
-    if (!mbar_wait_suspended(empty_bar(s), ph ^ 1u, abort_flag)) { fail(abort_flag, plan().err, ERR_PRODUCER); failed = true; }
+    if (!warp_wait_suspended(empty_bar(s), ph ^ 1u, abort_flag)) { fail(abort_flag, plan().err, ERR_PRODUCER); failed = true; }
     // row k of a slice's atom: 128 bytes [pol X | pol Y][32 spectra], 16-byte chunks XOR (k & 7);
     // station s0 + 8 i holds rows k = 2 s0 + 16 i (re) and k + 1 (im).  (After an expired wait the
     // stage is overwritten all the same: the launch has failed.)
@@ -788,7 +788,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
       uint32_t k = 0;
       for (int item = blockIdx.x; item < L.items; item += gridDim.x, k ^= 1u) {
         const SpParams &p = L.plan[kMulti ? plan_of(L, item) : 0];
-        if (!mbar_wait_suspended(wfree, k ^ 1u, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); break; }
+        if (!warp_wait_suspended(wfree, k ^ 1u, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); break; }
         eval_weights(p, wstage, item_of(p, item), ew, lane);
         __syncwarp();
         if (lane == 0) mbar_arrive(wready);
@@ -821,7 +821,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
       const SpParams &pn = L.plan[kMulti ? plan_of(L, more ? ni : item) : 0];
       // the weights of item number k (of this CTA) to TMEM
       auto put = [&](const SpParams &q, int k) -> bool {
-        if (!mbar_wait(wready, (uint32_t)k & 1u, abort_flag)) { fail(abort_flag, q.err, ERR_EPILOGUE); return false; }
+        if (!warp_wait(wready, (uint32_t)k & 1u, abort_flag)) { fail(abort_flag, q.err, ERR_EPILOGUE); return false; }
         put_weights(q, wstage, tl + kW0, quad * 16 + jq, ro, half);
         tc_fence_before();
         __syncwarp();
@@ -835,16 +835,17 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
       for (int t = w.t0; t < w.t1; ++t, gpar ^= 1u) {
         float2 vx[16], vy[16];
         if (nb <= 0) {   // no beams in this lane quadrant: keep the barriers and the weights going
-          if (!mbar_wait(d2full, gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+          if (!warp_wait(d2full, gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
           if (lane == 0) mbar_arrive(d2empty);
-          if (!mbar_wait(d1full, gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+          if (!warp_wait(d1full, gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+          tc_fence_after();   // put() overwrites the weights that the MMAs of D1 have read
           if (t == w.t1 - 1 && more && !put(pn, eit + 1)) { ok = false; break; }
           if (lane == 0) mbar_arrive(d1empty);
           bad |= nonfinite[slot * 2] | nonfinite[slot * 2 + 1];
           slot = (slot + 1) & (kSlots - 1);
           continue;
         }
-        if (!mbar_wait(d2full, gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+        if (!warp_wait(d2full, gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
         tc_fence_after();
         {
           float a[2][16], d[2][16];
@@ -863,7 +864,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(d2empty);
-        if (!mbar_wait(d1full, gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+        if (!warp_wait(d1full, gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
         tc_fence_after();
         // every MMA that reads this item's weights is complete
         if (t == w.t1 - 1 && more && !put(pn, eit + 1)) { ok = false; break; }
@@ -906,7 +907,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
             if ((t + 1) % St::kPeriod == 0 || t == w.t1 - 1) {
               __syncwarp();
               if (lane == 0) mbar_arrive(pair_bar(quad));
-              if (!mbar_wait(pair_bar(quad), (uint32_t)fl & 1u, abort_flag)) {
+              if (!warp_wait(pair_bar(quad), (uint32_t)fl & 1u, abort_flag)) {
                 fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break;
               }
               flush_stage<NS, Q>(p, buf, half * 32 + lane, quad, w.bb, f, c, wbase);
@@ -918,7 +919,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
       if (ok && bad) {   // the same value in every epilogue warp; all of them have stored the item first
         __syncwarp();
         if (lane == 0) mbar_arrive(fix_bar);
-        if (!mbar_wait(fix_bar, fpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); break; }
+        if (!warp_wait(fix_bar, fpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); break; }
         fpar ^= 1u;
         fix_item<NS, Q>(p, w, tid - 128);
       }

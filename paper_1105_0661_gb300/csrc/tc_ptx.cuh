@@ -78,6 +78,30 @@ __device__ __forceinline__ bool mbar_wait_suspended(uint32_t bar, uint32_t parit
   }
 }
 
+// The waits of a whole warp: one answer for all lanes, which have converged again when it returns.  A
+// lane still polling while lane 0 went on and arrived elsewhere could miss its phase (the parity comes
+// back two phases later), and the .sync.aligned tensor-memory instructions need the whole warp.  The
+// vote sits in the loop: behind the loops above it cost the epilogue registers (spills, 5-14 %).
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+  for (uint32_t i = 0; i < kWaitIters; ++i) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (__all_sync(0xffffffffu, done)) return true;
+    if (__any_sync(0xffffffffu, *abort_flag)) return false;
+    if (i > 64) __nanosleep(64);
+  }
+  return false;
+}
+__device__ __forceinline__ bool warp_wait_suspended(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait_suspended(bar, parity, abort_flag));
+}
+
 __device__ __forceinline__ void fail(volatile int *abort_flag, int *err, int code) {
   *abort_flag = 1;
   atomicCAS(err, 0, code);

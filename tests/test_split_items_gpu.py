@@ -1,0 +1,49 @@
+"""The split beam former over several work items per CTA with lane quadrants that hold no beams (the last
+64-beam block of 33, 49 or 80 beams): the weights of one item follow another's in tensor memory while
+those warps only keep the barriers going.
+
+Bound: a weight and a sample component are off by at most 2^-24 of 1 and of the column's peak each,
+which over the real and imaginary parts of S stations stays below 8e-7 x S x peak."""
+
+import numpy as np
+import pytest
+
+from oracle import lbf_oracle as O
+from synth import generate as G
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+N = 256
+
+
+@pytest.mark.parametrize("S,B,M,Q,out", [(24, 33, 128, 1, "V"), (16, 49, 64, 8, "I"), (24, 80, 192, 4, "IQUV"),
+                                         (40, 33, 64, 16, "IQUV")])
+def test_quadrants_without_beams(S, B, M, Q, out):
+    from paper_1105_0661_gb300 import Plan, build_lib
+    build_lib.build()
+    dev = torch.device("cuda:0")
+    F = 4                                            # 1024 or 2048 items
+    rng = np.random.default_rng(S + B)
+    wl = G.Workload("items", G.lofar_positions(rng, S // 2, S - S // 2), G.subband_centres(F, 120e6),
+                    G.hex_beam_grid(B, 0.05), (0.3, 0.4), M * N, Q, out)
+    shape = (F, N, S, 2, M)
+    ct = (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+    x = torch.from_numpy(ct).to(dev)
+    p = Plan.from_workload(wl)
+    ob = O.observation_from_workload(wl)
+    v = ob.beamform(ct.astype(np.complex128))
+    dv = 8e-7 * S * np.abs(ct).max()
+    for _ in range(3):
+        if out == "V":
+            o = torch.full(p.shape("vol"), float("nan"), dtype=torch.complex64, device=dev)
+            p.beamform(x, o)
+            assert np.abs(o.cpu().numpy() - v).max() <= dv
+        else:
+            o = torch.full(p.shape("stokes"), float("nan"), dtype=torch.float32, device=dev)
+            p.beamform_stokes(x, o)
+            ref = ob.stokes(v)
+            # |dI| <= 2 |V| |dV| + |dV|^2 summed over pols and spectra
+            assert np.all(np.abs(o.cpu().numpy() - ref) <= 4 * dv * (ref[:, :1] * Q) ** 0.5 + 4e-7 * ref[:, :1])
+        assert p.device_status() == 0
+    p.close()
