@@ -70,8 +70,10 @@ struct IncAcc {
 // (few_log_channels).  FB = 16 reads the corner-turned block half as often for 9 to 32 beams (16 FP32
 // flop per byte, about the FP32/HBM ridge).
 // kOne: lg is 0 (known to the compiler, which then keeps the item's pointers in uniform registers).
+// ct is not __restrict__: behind a programmatic launch the filter bank still writes the block while this
+// kernel is resident, and the promise would allow non-coherent loads, also ahead of wait_for_previous.
 template <int OUT, int FB, bool kOne>
-__device__ __forceinline__ void bf_few_item(const Geometry &g, const float2 *__restrict__ ct, void *__restrict__ out,
+__device__ __forceinline__ void bf_few_item(const Geometry &g, const float2 *ct, void *__restrict__ out,
                                             int fc0, int lg, int bgrp, float2 *wsm /* [2^lg][S][FB] */) {
   const int b0 = bgrp * FB;
   const int lt = kOne ? 8 : 8 - lg;           // log2 of the threads of a channel
@@ -158,7 +160,7 @@ __device__ __forceinline__ void bf_few_item(const Geometry &g, const float2 *__r
 // the Stokes I time
 template <int OUT, int FB, bool kOne>
 __global__ void __launch_bounds__(kFewThreads, (OUT == OUT_STOKES_I && FB == 8) ? 3 : 2)
-bf_few_kernel(Geometry g, const float2 *__restrict__ ct, void *__restrict__ out, int lg) {
+bf_few_kernel(Geometry g, const float2 *ct, void *__restrict__ out, int lg) {
   extern __shared__ __align__(16) float2 wsm[];
   bf_few_item<OUT, FB, kOne>(g, ct, out, blockIdx.x, lg, blockIdx.y, wsm);
 }

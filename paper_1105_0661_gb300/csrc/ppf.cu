@@ -256,8 +256,8 @@ __device__ __forceinline__ void ppf_drain(PpfCtl &c) {
 // kStall: failure-detection test build, the item issues none of its input copies (its waits
 // expire); launched only when the test asks for it, so the production kernels are untouched.
 template <int BITS, int MODE, bool kTmaSt, bool kStall = false>
-__device__ __forceinline__ void ppf_item(const Geometry &g, const typename SampleIO<BITS>::word *__restrict__ in,
-                                         const typename SampleIO<BITS>::word *__restrict__ hist, const PpfOut &po,
+__device__ __forceinline__ void ppf_item(const Geometry &g, const typename SampleIO<BITS>::word *in,
+                                         const typename SampleIO<BITS>::word *hist, const PpfOut &po,
                                          int s, int f, int chunk, int spc, PpfSmem<BITS> &sm, uint32_t &ph,
                                          const PpfMaps *maps) {
   using word = typename SampleIO<BITS>::word;
@@ -618,8 +618,7 @@ __device__ __forceinline__ void ppf_item(const Geometry &g, const typename Sampl
 // The next block's history of stream sf, samples [e0, e1): the last H samples of [history | block].
 template <typename word>
 __device__ __forceinline__ void copy_history(const Geometry &g, long long sf, int e0, int e1, int tid, int threads,
-                                             const word *__restrict__ in, const word *__restrict__ hist,
-                                             word *__restrict__ nhist) {
+                                             const word *in, const word *hist, word *__restrict__ nhist) {
   const word *h = hist + sf * g.H + g.T, *x = in + sf * g.T + (g.T - g.H);
   word *d = nhist + sf * g.H;
   const int cut = g.H - g.T;                  // samples before `cut` come from the old history
@@ -627,11 +626,13 @@ __device__ __forceinline__ void copy_history(const Geometry &g, long long sf, in
   for (int e = e0 + tid; e < e1; e += threads) d[e] = e < cut ? h[e] : x[e];
 }
 
-// kHist: the CTA also writes its share of the next block's history (nhist).
+// kHist: the CTA also writes its share of the next block's history (nhist).  in and hist are not
+// __restrict__: in a programmatic launch the kernels before may still write them while this one is
+// resident, and the promise would allow non-coherent loads, also ahead of wait_for_previous.
 template <int BITS, int MODE, bool kTma, bool kHist, bool kStall = false>
 __global__ void __launch_bounds__(kThreads, 1)
-ppf_kernel(Geometry g, const typename SampleIO<BITS>::word *__restrict__ in,
-           const typename SampleIO<BITS>::word *__restrict__ hist, typename SampleIO<BITS>::word *__restrict__ nhist,
+ppf_kernel(Geometry g, const typename SampleIO<BITS>::word *in,
+           const typename SampleIO<BITS>::word *hist, typename SampleIO<BITS>::word *__restrict__ nhist,
            PpfOut po, int chunks, int spc, const __grid_constant__ PpfMaps maps) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // The tensor stores read 128-byte-aligned staging buffers: the layout aligns them within itself
