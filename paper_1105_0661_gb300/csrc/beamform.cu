@@ -181,7 +181,7 @@ cudaError_t launch_few(const Geometry &g, int out_kind, const float2 *ct, void *
   dim3 grid((unsigned)((g.F * kN) >> lg), (unsigned)((g.B + fb - 1) / fb));
   const size_t smem = ((size_t)g.S * fb * sizeof(float2)) << lg;
   auto go = [&](auto kern) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_behind(g.pdl != 0, kern, grid, kFewThreads, smem, st, g, ct, out, lg);
   };
@@ -433,7 +433,7 @@ cudaError_t launch_many(const Geometry &g, int out_kind, const float2 *ct, void 
   const long long ctas = (long long)g.F * kN * nbt;
   const size_t smem = (size_t)g.S * (BT + 2 * kP * kMC) * sizeof(float2);
   auto go = [&](auto kern) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)ctas, kManyThreads, smem, st>>>(g, ct, out, nbt);
     return cudaGetLastError();
@@ -543,11 +543,13 @@ cudaError_t launch_beamform(const Geometry &g, int variant, int out_kind, const 
 
 namespace {
 
+constexpr size_t kGroupStatic = 16;   // bf_group_kernel's item_s and grp_s
+
 template <int V, int OUT>
 cudaError_t launch_group_t(const BfTable &T, long long total, unsigned long long *counter, size_t smem,
                            cudaStream_t st) {
   auto kern = bf_group_kernel<V, OUT>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared(kern, smem, kGroupStatic);
   if (e != cudaSuccess) return e;
   // persistent: as many CTAs as are resident at once (registers and this launch's shared memory)
   int per_sm = 0, dev = 0, sms = 0;
@@ -573,7 +575,7 @@ cudaError_t launch_group_v(int out_kind, const BfTable &T, long long total, unsi
 template <int V, int OUT>
 int residency_t(size_t smem) {
   auto kern = bf_group_kernel<V, OUT>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  if (allow_shared(kern, smem, kGroupStatic) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }

@@ -68,7 +68,7 @@ constexpr int kBarBytes = 1024;
 constexpr int kSlots = 8;                   // column-scale ring: more than the stages + 3 tiles in flight
 constexpr int kScaleBytes = kSlots * kCols * 4;
 constexpr int kColmaxBytes = 2 * 3 * 64 * 4;   // [group][3][column]
-constexpr int kSmemLimit = 227 * 1024;
+constexpr int kSmemLimit = (int)kCtaSharedBytes;
 // shared memory: barriers and flags, column scales, column maxima, stage ring (1024-byte aligned),
 // output staging, weight stage
 constexpr int kScaleOff = kBarBytes, kColmaxOff = kScaleOff + kScaleBytes;
@@ -959,7 +959,7 @@ cudaError_t launch_q(SpLaunch &L, int grid, cudaStream_t st) {
     return cudaFuncGetAttributes(&a, kern) == cudaSuccess ? a.numRegs : 0;
   }();
   if (regs < kLaunchRegs) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_shared(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<grid, kThreads, smem, st>>>(L);
   return cudaGetLastError();

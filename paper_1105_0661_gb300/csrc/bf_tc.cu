@@ -51,7 +51,7 @@ constexpr int kMTiles = 2;                  // 128 beams per work item
 constexpr int kBeamsPerItem = kMTiles * kRows / 2;
 constexpr int kMaxStages = 8;
 constexpr int kBarBytes = 1024;             // barriers, TMEM slot, flags
-constexpr int kSmemLimit = 227 * 1024;
+constexpr int kSmemLimit = (int)kCtaSharedBytes;
 constexpr int kRingBytes = kSmemLimit - 1024 /* alignment slack */ - kBarBytes;
 constexpr int kMinSmem = 120 * 1024;
 // TMEM: 2 accumulators of 128 columns + 2 x 2 weight planes of <= 64
@@ -733,7 +733,7 @@ cudaError_t launch_q(TcLaunch &L, int grid, cudaStream_t st) {
   // at least half of an SM's shared memory, so that no two CTAs share an SM (each holds all of
   // its TMEM columns)
   if (smem < kMinSmem) smem = kMinSmem;
-  cudaError_t e = cudaFuncSetAttribute(bf_tc_kernel<NS, Q, kForm>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_shared(bf_tc_kernel<NS, Q, kForm>, smem);
   if (e != cudaSuccess) return e;
   bf_tc_kernel<NS, Q, kForm><<<grid, tc_threads<NS, Q, kForm>(), smem, st>>>(L);
   return cudaGetLastError();

@@ -224,7 +224,7 @@ cudaError_t launch_dedisperse(const Geometry &g, double dm, int K, const float2 
     return cudaGetLastError();
   }
   const size_t smem = sizeof(float2) * ((size_t)K / 2 + K + (size_t)d.runs_per_pass * K);
-  cudaError_t e = cudaFuncSetAttribute(dedisperse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared(dedisperse_kernel, smem, 16 /* coef_s */);
   if (e != cudaSuccess) return e;
   dedisperse_kernel<<<(unsigned)ctas, kThreads, smem, st>>>(g, d, in, out);
   return cudaGetLastError();

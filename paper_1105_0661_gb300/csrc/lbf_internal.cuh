@@ -215,6 +215,17 @@ int many_beam_max_stations();
 cudaError_t launch_stokes(const Geometry &g, int out_kind, const float2 *vol, float *out,
                           cudaStream_t st);
 
+// Let `kern` take `smem` bytes of dynamic shared memory.  The limit belongs to the kernel, for every thread
+// of the process: each launch sets the same one, what a CTA may have at most beside the kernel's static
+// shared memory (at most `fixed` bytes), so that no thread lowers it between another's call here and
+// its launch.
+constexpr size_t kCtaSharedBytes = 227 * 1024;
+template <typename K>
+cudaError_t allow_shared(K kern, size_t smem, size_t fixed = 0) {
+  if (smem > kCtaSharedBytes - fixed) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kCtaSharedBytes - fixed));
+}
+
 // Launch `kern`; with `pdl` as a programmatic dependent launch: its CTAs may start while the kernel
 // before it on the stream still runs (once that has called let_dependents_start in every CTA, or has
 // ended), and must call wait_for_previous before they read or write what it writes or reads.  Saves a
