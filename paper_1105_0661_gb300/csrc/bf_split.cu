@@ -1,11 +1,11 @@
 // FP32 tied-array beam former (Section 4.3) on the tensor cores: the FP32 corner-turned block and
-// the weights are cut into FP16 slices, four slice products run as tcgen05 MMAs, and the result is
-// at least as close to the 64-bit value as that of the FP32 FMA kernels of beamform.cu.  Fused with
-// the Stokes I / IQUV integration epilogue (Sections 4.5, 5.1) or writing the beam voltages.
+// the weights are cut into FP16 slices, six slice products run as tcgen05 MMAs, and the result is no
+// further from the 64-bit value than that of the FP32 FMA kernels of beamform.cu.  Fused with the
+// Stokes I / IQUV integration epilogue (Sections 4.5, 5.1) or writing the beam voltages.
 //
 // Why: the beam former of B beams does 16 B flop per station-sample.  In FP32 FMAs that is bound by
 // the FMA pipe from about 10 beams on (80 TFLOP/s: 58 ms for the 127-beam LOFAR block), while the
-// block could be read in 5.4 ms and its four FP16 products take 8 ms at the tensor-core rate.
+// block could be read in 5.4 ms and its six FP16 products take 12 ms at the tensor-core rate.
 //
 // The slices.  The tensor cores add FP16 products exactly but truncate the FP32 accumulator toward
 // zero as they go; that bias does not average out over an integration window, and is why the
@@ -13,18 +13,21 @@
 // error-free transformation of Ozaki, Ogita, Oishi and Rump, Numerical Algorithms 59, 2012):
 //  * a column of the block (one spectrum and polarisation, all stations) is scaled by the power of
 //    two that puts its largest component in [2^10, 2^11); y1 is the scaled value rounded to an
-//    integer and y2 = fp16(the rest);
-//  * 128 w = w1 + w2 + w3 with w1 an integer, w2 and w3 FP16 (exact to 2^-29), w12 = fp16(128 w);
-//  * D1 = W1 Y1 sums integers up to 2^18, which stay below 2^24 even if all 64 stations are in
-//    phase, so D1 never rounds; D2 = W2 Y1 + W3 Y1 + W12 Y2 accumulates apart from it, 2^7 smaller
-//    and more, so that its truncation is below the result's last bit;
+//    integer, y2 the rest rounded to a multiple of 2^-11 and y3 what then remains in FP16, good to
+//    2^-34 of the peak: a station a thousand times weaker than the strongest keeps its 24 bits;
+//  * 128 w = w1 + w2 + w3 with w1 an integer, w2 and w3 FP16 (exact to 2^-29);
+//  * D1 = W1 Y1 sums integers up to 2^18.5 and rounds nothing; D2 = W2 Y1 + W3 Y1 + W1 Y2 + W2 Y2 +
+//    W1 Y3 accumulates apart from it, 2^7 smaller and more, so that its truncation is below the
+//    result's last bit; the products left out are below 2^-31 of the peak;
 //  * V = (D1 + D2) 2^-e in FP32.
-// What remains is the rounding of y2 (2^-24 of the column's peak) and of w12 in W12 Y2 (6e-8), where
-// the FMA kernels round the accumulator at every station.  Relative RMS error against 64 bits, FMA
-// kernels and this one: beam voltages of 24 stations 1.8e-7 and 1.8e-7 (1.3e-7 of it the filter
-// bank's), of 48 stations after dedispersion 2.7e-7 and 2.4e-7, Stokes I of the LOFAR block 6.9e-8
-// and 6.7e-8, unintegrated IQUV 1.8e-7 and 8e-8.  Columns that hold an infinity are recomputed at the
-// end of their work item with FP32 FMAs (fix_item).
+// What remains is the rounding of V and of the FP32 weights, where the FMA kernels round the
+// accumulator at every station.  RMS error of the voltages against 64 bits for a given block, FMA
+// kernel and this one: 8 stations 7.5e-8 and 3.7e-8, 24 stations 1.2e-7 and 3.6e-8, 64 stations 2.0e-7
+// and 3.6e-8; 48 stations with the first 30 times stronger 2.4e-7 and 3.7e-8, with the last 5.6e-8 and
+// 4.0e-8.  (Two slices of y and w12 = fp16(128 w) in the place of the last three products are off by
+// 1.2e-7 to 1.5e-7 for equal stations, but by 4.4e-7 in the last two cases: 127 beams of 30 subbands
+// took 2.0 ms so, 2.5 with three slices.)  Columns that hold an infinity are recomputed at the end of
+// their work item with FP32 FMAs (fix_item).
 //
 // Work.  A persistent CTA per SM walks the work items (f, c, span of spectra, block of 64 beams)
 // with a stride of the grid; the beam blocks of one (f, c) run together and share its block in L2.
@@ -34,19 +37,21 @@
 //  * converter warps (8, two groups of four; a group owns one 32-spectrum half of each tile): each
 //    thread loads four adjacent spectra of one polarisation of every eighth station (one 32-byte load
 //    where rows allow it), the column maxima meet in shared memory across a barrier of the group, and
-//    the two slices go to the stage ring in the swizzled layout the MMA reads (64-bit stores, a whole
+//    the three slices go to the stage ring in the swizzled layout the MMA reads (64-bit stores, a whole
 //    128-byte row per half-warp: no bank conflicts).  The loads of the next tile are issued as the
 //    registers of the current one are consumed; the MMA thread prefetches the tiles after it into L2
 //    (one tensor box per tile: a row at a time from the converters, the prefetches took 2700 cycles
 //    per tile).  Sixteen warps of two spectra per thread: 10 % slower (twice the loop overhead).
 //  * epilogue warps (8): warp w serves TMEM lane quadrant w % 4 and one 32-spectrum half.  They take
 //    D2 into registers while the MMAs fill D1, and D1 while the MMAs fill the next tile's D2, so
-//    that one accumulator of each suffices (256 TMEM columns, next to 4 x 64 of weight slices).
-// What bounds it: the issue slots (ncu, 8 subbands of the LOFAR block: 57 % of them used, 7300 warp
-// instructions per tile of 64 beams, half of them the converters', a quarter the epilogue's) and the
-// latency of the converters' chain; the MMAs take half of a tile's 3300 cycles.  127 beams of the
-// LOFAR block: 86.2 ms in FP32 FMAs, 16.5 here; 37 beams of 30 subbands: 5.5 ms and 1.07; voltages of
-// 127 beams, 16 subbands: 5.7 ms and 1.8.
+//    that one accumulator of each suffices (256 TMEM columns, next to 3 x 64 of weight slices).
+// What bounds it: the latency of the converters' chain and the issue slots; the MMAs (64 cycles each)
+// take 2300 of a tile's 4000 cycles at 48 stations.  127 beams of the LOFAR block: 86.2 ms in FP32
+// FMAs, 20.5 here; 37 beams of 30 subbands: 5.5 ms and 1.29; voltages of 127 beams, 16 subbands: 5.7 ms
+// and 1.87.  The ring holds two stages up to 56 stations and one beyond (64 stations, 127 beams, 8
+// subbands: 1.20 ms against 0.74 for 56).  Measured and dropped: stages of two slices that share a third
+// one (64 stations 1.20 -> 1.10 ms, 48 stations 0.67 -> 0.71: registers), stages released by halves (an
+// MMA of 64 columns takes as long as one of 128: 48 stations 0.67 -> 1.08).
 // Every mbarrier wait is bounded: on expiry the kernel records an error code, stops issuing work,
 // waits (bounded) for its MMAs in flight, frees TMEM and returns.  The MMA thread, the evaluators and
 // the converters wait suspended; the epilogue polls (suspended waits cost it up to 70 % on short
@@ -77,20 +82,22 @@ constexpr int kGfailOff = 232, kAbortOff = 228;
 constexpr int kRingOff = (kColmaxOff + kColmaxBytes + 1023) / 1024 * 1024;
 constexpr int kFixed = 1024 /* alignment slack */ + kRingOff;
 constexpr int kMinSmem = 120 * 1024;        // one CTA per SM: each allocates all of TMEM
-constexpr uint32_t kD1 = 0, kD2 = kCols, kW0 = 2 * kCols;   // TMEM columns: D1, D2, four weight slices
+constexpr uint32_t kD1 = 0, kD2 = kCols, kW0 = 2 * kCols;   // TMEM columns: D1, D2, three weight slices
 constexpr uint32_t kWPlane = 64;
 constexpr float kWUnit = 128.f;
 constexpr float kMagic = 12582912.f;        // 1.5 * 2^23: x + kMagic rounds x to an integer
+constexpr float kMagic2 = 6144.f;           // 1.5 * 2^12: x + kMagic2 rounds x to a multiple of 2^-11
 constexpr int kPrefetch = 4;                // tiles an L2 prefetch runs ahead of the loads
 // registers per thread after the split of what the CTA is launched with (640 x 96 = 61440):
-// 128 x 40 + 256 x 120 + 256 x 96 = 60416
+// 128 x 40 + 256 x 112 + 256 x 104 = 60416.  The compiler allocates each section by its own share: with
+// 96 for the converters of three slices all kernels spilled 300 bytes and more a thread, with 104 up to 40
 constexpr int kLaunchRegs = 96;
 
 struct SpParams {
   int S, F, B, M, Kpad, ntiles, ipf;        // ipf: beam blocks per (f, c)
   int tpc, chunks;                          // tiles per item, items along the spectra
   int items, first_item;
-  int stage_bytes;                          // 2 slices x 2 atoms x Kpad rows x 128 bytes
+  int stage_bytes;                          // 3 slices x 2 atoms x Kpad rows x 128 bytes
   int vec, align;                           // output rows 16-byte aligned; bytes the input rows are aligned to
   const int *phase0;
   const float *step;
@@ -134,12 +141,13 @@ __device__ __forceinline__ float2 weight_of(const SpParams &p, int f, int c, int
                                    (float)(c - kN / 2)));
 }
 
-// The weights of an item go through the weight stage [slice][S][64 beams] in shared memory, one
-// half2 (cos, sin) per slice: 128 w = w1 + w2 + w3 with w1 an integer and w2, w3 FP16 (fp16(128 w) =
-// fp16(w1 + w2) is formed on the way to TMEM).  The evaluator warps fill it while the item before
-// runs; the epilogue warps move it to TMEM (put_weights) as soon as that item's last MMA is done.
+// The weights of an item go through the weight stage [S][64 beams] float2 in shared memory.  The
+// evaluator warps fill it while the item before runs; the epilogue warps slice them on their way to
+// TMEM (put_weights) as soon as that item's last MMA is done.  (Sliced by the evaluators, the stage is
+// half as large again, and IQUV of 52 to 56 stations keeps one ring stage: 8 subbands, 127 beams 1.14 ms
+// against 0.79.)
 constexpr int kEvalWarps = 3;
-constexpr int weight_stage_bytes(int Kpad) { return 3 * (Kpad / 2) * kItemBeams * 4; }
+constexpr int weight_stage_bytes(int Kpad) { return (Kpad / 2) * kItemBeams * 8; }
 
 // exp(2 pi i phi) of two phases in 2^-32 cycle, as packed operations: reduced to the nearest quarter
 // cycle in integers, then the Taylor polynomials of sine (degree 9) and cosine (degree 10), whose
@@ -181,7 +189,7 @@ __device__ __forceinline__ void slice_weight(float2 w, uint32_t &w1, uint32_t &w
 
 // Beams fastest over the lanes of a warp, so that the stage is written without bank conflicts; a
 // lane keeps one beam and walks the stations.
-__device__ __forceinline__ void eval_weights(const SpParams &p, uint32_t *stage, const Item &it, int ew, int lane) {
+__device__ __forceinline__ void eval_weights(const SpParams &p, float2 *stage, const Item &it, int ew, int lane) {
   const int f = it.fc / kN, S2 = p.Kpad / 2;
   const float dc = (float)(it.fc - f * kN - kN / 2);
 #pragma unroll 1
@@ -201,8 +209,7 @@ __device__ __forceinline__ void eval_weights(const SpParams &p, uint32_t *stage,
       for (int e = 0; e < 2; ++e) {
         const int s = s0 + k + e;
         if (b >= p.B || s >= p.S) w[e] = make_float2(0.f, 0.f);
-        uint32_t *d = stage + s * kItemBeams + bl;
-        slice_weight(w[e], d[0], d[S2 * kItemBeams], d[2 * S2 * kItemBeams]);
+        stage[s * kItemBeams + bl] = w[e];
       }
     }
   }
@@ -210,30 +217,22 @@ __device__ __forceinline__ void eval_weights(const SpParams &p, uint32_t *stage,
 
 // Column s of a slice in TMEM holds (Re w, -Im w) for a Re row (ro = 0) and (Im w, Re w) for an Im
 // row; warp `half` of a lane quadrant moves every second group of 8 stations.  bl: beam of the row.
-__device__ __forceinline__ void put_weights(const SpParams &p, const uint32_t *stage, uint32_t ta, int bl, int ro,
+__device__ __forceinline__ void put_weights(const SpParams &p, const float2 *stage, uint32_t ta, int bl, int ro,
                                             int half) {
-  const int S2 = p.Kpad / 2;
   const uint32_t sel = ro ? 0x1032u : 0x3210u, flip = ro ? 0u : 0x80000000u;
 #pragma unroll 1
   for (int g8 = half; g8 < p.Kpad / 16; g8 += 2) {
-    const uint32_t *d = stage + g8 * 8 * kItemBeams + bl;
+    const float2 *d = stage + g8 * 8 * kItemBeams + bl;
     const uint32_t t = ta + (uint32_t)(g8 * 8);
-    uint32_t a[8], b[8];
+    uint32_t a[3][8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      a[j] = __byte_perm(d[j * kItemBeams], 0, sel) ^ flip;
-      b[j] = __byte_perm(d[(S2 + j) * kItemBeams], 0, sel) ^ flip;
-    }
-    tmem_st8(t, a);
-    tmem_st8(t + kWPlane, b);
+      slice_weight(d[j * kItemBeams], a[0][j], a[1][j], a[2][j]);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const __half2 w12 = __hadd2(*reinterpret_cast<const __half2 *>(&a[j]), *reinterpret_cast<const __half2 *>(&b[j]));
-      a[j] = *reinterpret_cast<const uint32_t *>(&w12);
-      b[j] = __byte_perm(d[(2 * S2 + j) * kItemBeams], 0, sel) ^ flip;
+      for (int k = 0; k < 3; ++k) a[k][j] = __byte_perm(a[k][j], 0, sel) ^ flip;
     }
-    tmem_st8(t + 2 * kWPlane, b);
-    tmem_st8(t + 3 * kWPlane, a);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) tmem_st8(t + k * kWPlane, a[k]);
   }
   tmem_wait_st();
 }
@@ -619,7 +618,7 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
     unsigned char *re = sbase + kRingOff + (size_t)s * L.stage_max + (size_t)grp * (Kpad * 128) + k0 * 128 + within;
     unsigned char *im = re + 128 + ((chunk ^ (uint32_t)((k0 + 1) & 7)) << 4);
     re += (chunk ^ (uint32_t)(k0 & 7)) << 4;
-    const uint32_t lo_off = (uint32_t)Kpad * 256;
+    const uint32_t slice = (uint32_t)Kpad * 256;
     // on to the next tile
     ptr += kTileSpec;
     if (++t == t1) {
@@ -628,21 +627,25 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
       if (more) enter();
     }
     const int nS = more ? plan().S : 0, nM = plan().M;
-    const float2 mg = make_float2(kMagic, kMagic), m1 = make_float2(-1.f, -1.f);
+    const float2 mg = make_float2(kMagic, kMagic), mg2 = make_float2(kMagic2, kMagic2), m1 = make_float2(-1.f, -1.f);
 #pragma unroll
     for (int i = 0; i < NLD; ++i) {
-      float2 h[4], l[4];
+      float2 h[4], m[4], l[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const float2 x = make_float2(r[i][2 * e], r[i][2 * e + 1]), sx = make_float2(sc[e], sc[e]);
-        h[e] = __ffma2_rn(__ffma2_rn(x, sx, mg), m1, mg);   // minus the leading slice
+        h[e] = __ffma2_rn(__ffma2_rn(x, sx, mg), m1, mg);   // minus the first slice
         l[e] = __ffma2_rn(x, sx, h[e]);
+        m[e] = __ffma2_rn(__fadd2_rn(l[e], mg2), m1, mg2);   // minus the second
+        l[e] = __fadd2_rn(l[e], m[e]);
       }
       if (i < steps) {
         *reinterpret_cast<uint2 *>(re + i * (kGroup * 512)) = make_uint2(pack_half2(-h[0].x, -h[1].x), pack_half2(-h[2].x, -h[3].x));
         *reinterpret_cast<uint2 *>(im + i * (kGroup * 512)) = make_uint2(pack_half2(-h[0].y, -h[1].y), pack_half2(-h[2].y, -h[3].y));
-        *reinterpret_cast<uint2 *>(re + lo_off + i * (kGroup * 512)) = make_uint2(pack_half2(l[0].x, l[1].x), pack_half2(l[2].x, l[3].x));
-        *reinterpret_cast<uint2 *>(im + lo_off + i * (kGroup * 512)) = make_uint2(pack_half2(l[0].y, l[1].y), pack_half2(l[2].y, l[3].y));
+        *reinterpret_cast<uint2 *>(re + slice + i * (kGroup * 512)) = make_uint2(pack_half2(-m[0].x, -m[1].x), pack_half2(-m[2].x, -m[3].x));
+        *reinterpret_cast<uint2 *>(im + slice + i * (kGroup * 512)) = make_uint2(pack_half2(-m[0].y, -m[1].y), pack_half2(-m[2].y, -m[3].y));
+        *reinterpret_cast<uint2 *>(re + 2 * slice + i * (kGroup * 512)) = make_uint2(pack_half2(l[0].x, l[1].x), pack_half2(l[2].x, l[3].x));
+        *reinterpret_cast<uint2 *>(im + 2 * slice + i * (kGroup * 512)) = make_uint2(pack_half2(l[0].y, l[1].y), pack_half2(l[2].y, l[3].y));
       }
       if (kMulti) clear(i);                   // the next plan may have fewer stations
       load_tile(i, nS, nM);
@@ -674,7 +677,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
   unsigned char *after = sbase + kRingOff + (size_t)nst * L.stage_max;
   const float *const scales = reinterpret_cast<const float *>(sbase + kScaleOff);   // [kSlots][kCols]
   float *const stage_out = reinterpret_cast<float *>(after);
-  uint32_t *const wstage = reinterpret_cast<uint32_t *>(after + St::kBytes);
+  float2 *const wstage = reinterpret_cast<float2 *>(after + St::kBytes);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 64u + 8u * s; };
   const uint32_t d1full = bar0 + 128u, d1empty = bar0 + 136u, d2full = bar0 + 144u, d2empty = bar0 + 152u;
@@ -748,7 +751,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
         err = p.err;
         const Item w = item_of(p, item);
         const int ksteps = p.Kpad >> 4;
-        const uint64_t plane = (uint64_t)((uint32_t)p.stage_bytes >> 5);   // lo slice: half a stage on, / 16
+        const uint64_t slice = (uint64_t)((uint32_t)(p.Kpad * 256) >> 4);   // to the next slice of the block, / 16
         const uint64_t desc0 = smem_desc(sB, (uint32_t)(p.Kpad * 128));
         const uint32_t a0 = tmem + kW0;
         if (!mbar_wait_suspended(wfull, (uint32_t)it & 1u, abort_flag)) { fail(abort_flag, err, ERR_MMA); break; }
@@ -758,12 +761,14 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
           }
           tc_fence_after();
           const uint64_t b0 = desc0 + (uint64_t)((uint32_t)(s * L.stage_max) >> 4);
-          for (int ks = 0; ks < ksteps; ++ks) {      // D2 = W2 Y1 + W3 Y1 + W12 Y2
+          for (int ks = 0; ks < ksteps; ++ks) {      // D2 = W2 Y1 + W3 Y1 + W1 Y2 + W2 Y2 + W1 Y3
             const uint64_t b = b0 + (uint64_t)(ks * ((16 * 128) >> 4));
             const uint32_t a = a0 + 8u * ks;
             umma(tmem + kD2, a + kWPlane, b, ks != 0);
             umma(tmem + kD2, a + 2 * kWPlane, b, 1);
-            umma(tmem + kD2, a + 3 * kWPlane, b + plane, 1);
+            umma(tmem + kD2, a, b + slice, 1);
+            umma(tmem + kD2, a + kWPlane, b + slice, 1);
+            umma(tmem + kD2, a, b + 2 * slice, 1);
           }
           umma_commit(d2full);
           issued = true;
@@ -796,7 +801,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
     }
     __syncwarp();
   } else if (warp < 4 + kEpiWarps) {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
     // ---------------------------------------------------------------- epilogue
     const int ew = warp - 4, quad = warp & 3, half = ew >> 2;
     const int ro = lane & 1, jq = lane >> 1;
@@ -926,6 +931,7 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
     }
   } else {
     // ---------------------------------------------------------------- converters
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
     const int cw = warp - 4 - kEpiWarps;
     const int nld = L.plan[0].Kpad / 16, al = L.plan[0].align;
     if (kMulti || al == 8) convert<8, 8, kMulti>(L, sbase, cw, lane);
@@ -947,10 +953,10 @@ bf_split_kernel(const __grid_constant__ SpLaunch L) {
 template <int NS, int Q, bool kMulti>
 cudaError_t launch_q(SpLaunch &L, int grid, cudaStream_t st) {
   auto kern = bf_split_kernel<NS, Q, kMulti>;
-  const int wstage = weight_stage_bytes(L.stage_max / (4 * 128));   // of the largest Kpad
+  const int wstage = weight_stage_bytes(L.stage_max / (6 * 128));   // of the largest Kpad
   L.nstages = (kSmemLimit - kFixed - Stage<NS, Q>::kBytes - wstage) / L.stage_max;
   if (L.nstages > kMaxStages) L.nstages = kMaxStages;
-  if (L.nstages < 2) return cudaErrorInvalidValue;
+  if (L.nstages < 1) return cudaErrorInvalidValue;
   int smem = kFixed + L.nstages * L.stage_max + Stage<NS, Q>::kBytes + wstage;
   if (smem < kMinSmem) smem = kMinSmem;
   // the register split of the kernel's warpgroups draws on what the CTA was launched with
@@ -998,7 +1004,7 @@ bool fill_plan(SpLaunch &L, int i, const Geometry &g, int out_kind, const float2
   SpParams &p = L.plan[i];
   p.S = g.S; p.F = g.F; p.B = g.B; p.M = g.M;
   p.Kpad = ((2 * g.S + 15) / 16) * 16;
-  p.stage_bytes = 4 * p.Kpad * 128;
+  p.stage_bytes = 6 * p.Kpad * 128;
   p.ntiles = (g.M + kTileSpec - 1) / kTileSpec;
   p.ipf = (g.B + kItemBeams - 1) / kItemBeams;
   // whole (f, c) rows per item; an observation of few rows is cut along the spectra, in spans of
