@@ -12,13 +12,14 @@
 // three-product form of bf_tc.cu stays at 1e-6.  Here the leading product is exact instead (the
 // error-free transformation of Ozaki, Ogita, Oishi and Rump, Numerical Algorithms 59, 2012):
 //  * a column of the block (one spectrum and polarisation, all stations) is scaled by the power of
-//    two that puts its largest component in [2^10, 2^11); y1 is the scaled value rounded to an
+//    two that puts its largest component in [2^9, 2^10); y1 is the scaled value rounded to an
 //    integer, y2 the rest rounded to a multiple of 2^-11 and y3 what then remains in FP16, good to
-//    2^-34 of the peak: a station a thousand times weaker than the strongest keeps its 24 bits;
+//    2^-33 of the peak: a station 500 times weaker than the strongest keeps its 24 bits;
 //  * 128 w = w1 + w2 + w3 with w1 an integer, w2 and w3 FP16 (exact to 2^-29);
-//  * D1 = W1 Y1 sums integers up to 2^18.5 and rounds nothing; D2 = W2 Y1 + W3 Y1 + W1 Y2 + W2 Y2 +
-//    W1 Y3 accumulates apart from it, 2^7 smaller and more, so that its truncation is below the
-//    result's last bit; the products left out are below 2^-31 of the peak;
+//  * D1 = W1 Y1 never rounds: |w1| < 2^7.01 and |y1| <= 2^10.5 keep a station's term below 2^17.51 and
+//    the sum of 64 stations in phase below 2^23.51; D2 = W2 Y1 + W3 Y1 + W1 Y2 + W2 Y2 + W1 Y3
+//    accumulates apart from it, 2^7 smaller and more, so that its truncation is below the result's
+//    last bit; the products left out are below 2^-30 of the peak;
 //  * V = (D1 + D2) 2^-e in FP32.
 // What remains is the rounding of V and of the FP32 weights, where the FMA kernels round the
 // accumulator at every station.  RMS error of the voltages against 64 bits for a given block, FMA
@@ -599,12 +600,12 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
     const bool inf = group_sync_any(1 + grp, 32 * kGroup,
                                     fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) > 3.402823466e38f);
     if (gfail[grp * 2 + (n & 1)]) break;      // the whole group leaves together
-    // scale 2^(137 - E) for a peak in [2^(E - 127), 2^(E - 126)), E >= 10: the peak lands in
-    // [2^10, 2^11); its inverse, with the weights' 2^7, is 2^(E - 127) 2^-17
+    // scale 2^(136 - E) for a peak in [2^(E - 127), 2^(E - 126)), E >= 9: the peak lands in
+    // [2^9, 2^10); its inverse, with the weights' 2^7, is 2^(E - 127) 2^-16
     auto scale_of = [](uint32_t cb, float &inv) {
-      const uint32_t e = max(cb & 0x7f800000u, 10u << 23);
-      inv = __uint_as_float(e) * 7.62939453125e-6f;
-      return __uint_as_float((264u << 23) - e);
+      const uint32_t e = max(cb & 0x7f800000u, 9u << 23);
+      inv = __uint_as_float(e) * 1.52587890625e-5f;
+      return __uint_as_float((263u << 23) - e);
     };
     float4 inv;
     const float sc[4] = {scale_of(cm[0], inv.x), scale_of(cm[16], inv.y), scale_of(cm[32], inv.z),
