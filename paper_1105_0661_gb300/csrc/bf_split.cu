@@ -27,8 +27,8 @@
 // and 3.6e-8; 48 stations with the first 30 times stronger 2.4e-7 and 3.7e-8, with the last 5.6e-8 and
 // 4.0e-8.  (Two slices of y and w12 = fp16(128 w) in the place of the last three products are off by
 // 1.2e-7 to 1.5e-7 for equal stations, but by 4.4e-7 in the last two cases: 127 beams of 30 subbands
-// took 2.0 ms so, 2.5 with three slices.)  Columns that hold an infinity are recomputed at the end of
-// their work item with FP32 FMAs (fix_item).
+// took 2.0 ms so, 2.5 with three slices.)  Columns that hold an infinity, or nothing but numbers
+// below 2^-118, are recomputed at the end of their work item with FP32 FMAs (fix_item).
 //
 // Work.  A persistent CTA per SM walks the work items (f, c, span of spectra, block of 64 beams)
 // with a stride of the grid; the beam blocks of one (f, c) run together and share its block in L2.
@@ -426,8 +426,9 @@ __device__ __forceinline__ void voltage_half(const float2 (&vx)[16], const float
   }
 }
 
-// Recompute an item whose columns hold an infinity or a NaN with FP32 FMAs, station by station, as
-// the FMA kernels do (an infinite sample times a weight slice would turn into a NaN otherwise).
+// Recompute an item that has a column with an infinity or too small to scale with FP32 FMAs, station by
+// station, as the FMA kernels do (an infinite sample times a weight slice would turn into a NaN
+// otherwise).
 template <int NS, int Q>
 __device__ __noinline__ void fix_item(const SpParams &p, const Item &it, int et) {
   constexpr int kG = NS == 0 ? 4 : (Q < 4 ? 4 : Q);     // spectra per thread and step
@@ -608,8 +609,14 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
       return __uint_as_float((263u << 23) - e);
     };
     float4 inv;
-    const float sc[4] = {scale_of(cm[0], inv.x), scale_of(cm[16], inv.y), scale_of(cm[32], inv.z),
-                         scale_of(cm[48], inv.w)};
+    const uint4 peak = make_uint4(cm[0], cm[16], cm[32], cm[48]);
+    const float sc[4] = {scale_of(peak.x, inv.x), scale_of(peak.y, inv.y), scale_of(peak.z, inv.z),
+                         scale_of(peak.w, inv.w)};
+    // columns too small to scale (a peak below 2^-118, yet not zero) are left to the FMAs as well
+    auto tiny = [](uint32_t cb) { return cb - 1u < (9u << 23) - 1u; };
+    bool fix = inf;
+    if (wg == 0)   // the lanes of a warp cover the columns of the half tile
+      fix = __any_sync(0xffffffffu, inf || tiny(peak.x) || tiny(peak.y) || tiny(peak.z) || tiny(peak.w));
     if (!warp_wait_suspended(empty_bar(s), ph ^ 1u, abort_flag)) { fail(abort_flag, plan().err, ERR_PRODUCER); failed = true; }
     // row k of a slice's atom: 128 bytes [pol X | pol Y][32 spectra], 16-byte chunks XOR (k & 7);
     // station s0 + 8 i holds rows k = 2 s0 + 16 i (re) and k + 1 (im).  (After an expired wait the
@@ -653,7 +660,7 @@ __device__ __forceinline__ void convert(const SpLaunch &L, unsigned char *const 
     }
     if (!failed) {
       if (wg == 0 && lane < 16) *reinterpret_cast<float4 *>(scales + slot * kCols + grp * 64 + cc) = inv;
-      if (wg == 0 && lane == 0) nonfinite[slot * 2 + grp] = inf ? 1 : 0;
+      if (wg == 0 && lane == 0) nonfinite[slot * 2 + grp] = fix ? 1 : 0;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the slices visible to the MMA
       __syncwarp();
       if (lane == 0) mbar_arrive(full_bar(s));

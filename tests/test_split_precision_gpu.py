@@ -56,3 +56,11 @@ def test_no_further_from_64_bits_than_fp32_fmas(S, M, gain):
     split, fma = _rms(S, M, GAINS[gain](S))
     print(f"{S} stations, {gain}: split {split:.3e}, FMAs {fma:.3e}")
     assert split <= 1.05 * fma
+
+
+@pytest.mark.parametrize("scale", [1e-36, 1e-39])
+def test_small_and_denormal_columns(scale):
+    """Samples down to denormal numbers, too small for the power of two that scales a column."""
+    split, fma = _rms(24, 256, np.ones(24), scale)
+    print(f"scale {scale}: split {split:.3e}, FMAs {fma:.3e}")
+    assert split <= 1.05 * fma
