@@ -140,10 +140,10 @@ def algorithmic_work(wl, dims):
         "hist_update": ("hbm", 2 * S * F * dims.history_samples * word),
         "delay_ct": ("hbm", ss * 32),
         "bf_few": ("hbm", ss * 16 + out_bytes),  # read corner-turned cf32 once, write the output
-        # 8 flop per complex MAC, B x S x 2 pols x T per subband; up to 64 stations six FP16 slice
-        # products of the FP32 operands on the tensor cores, beyond that FP32 FMAs
-        "bf_many": ("tensor" if S <= 64 else "alu", 8.0 * B * ss * 2),
-        "bf_many64": ("tensor" if S <= 64 else "alu", 8.0 * B * ss * 2),
+        # 8 flop per complex MAC, B x S x 2 pols x T per subband
+        "bf_many": ("alu", 8.0 * B * ss * 2),
+        "bf_many64": ("alu", 8.0 * B * ss * 2),
+        "bf_split": ("tensor", 8.0 * B * ss * 2),   # six FP16 slice products of the FP32 operands
         "stokes": ("hbm", B * F * T * 16 + out_bytes),
         # FP16 forms: hi and lo half2 planes per pol; one complex product is the algorithmic work
         "ppf_ct16": ("hbm", ss * (word + 2 * 4 * 2)),
@@ -159,8 +159,8 @@ def traffic_from_profiles(kernel: str, workload_name: str):
     path = os.path.join(ROOT, "profiles", "traffic.md")
     if not os.path.exists(path):
         return None
-    src = {"bf_many": "bf_split.cu", "bf_many64": "bf_split.cu", "bf_few": "beamform.cu", "ppf_ct": "ppf.cu", "ppf": "ppf.cu",
-           "ppf_ct16": "ppf.cu", "bf_tc": "bf_tc.cu", "hist_update": "ppf.cu", "delay_ct": "delay.cu",
+    src = {"bf_many": "beamform.cu", "bf_many64": "beamform.cu", "bf_split": "bf_split.cu", "bf_few": "beamform.cu",
+           "ppf_ct": "ppf.cu", "ppf": "ppf.cu", "ppf_ct16": "ppf.cu", "bf_tc": "bf_tc.cu", "hist_update": "ppf.cu", "delay_ct": "delay.cu",
            "dedisperse": "dedisperse.cu",
            "stokes": "stokes.cu", "superstation": "delay.cu"}.get(kernel)
     if src is None:
@@ -690,8 +690,7 @@ def precision_form_1024(args, dev, stream, pk, smi_index):
                 ms = e0.elapsed_time(e1) / steps
                 r = {"ms_per_step": ms, "value": ss / (ms / 1e3), "steps": steps, "warmup": 3,
                      "kernels_ms": {k: v[1] / v[0] for k, v in tr.items() if not k.startswith("_") and v[0]}}
-                bf = "bf_tc" if prec != "fp32" else ("bf_many" if "bf_many" in r["kernels_ms"] else "bf_few")
-                bf_ms = r["kernels_ms"].get(bf)
+                bf_ms = next((t for k, t in r["kernels_ms"].items() if k.startswith("bf_")), None)
                 if bf_ms:
                     r["beamform_tflops"] = flop / (bf_ms / 1e3) / 1e12
                     if prec != "fp32":   # executed: three (fp16tc) or two (fp16tc2) FP16 products

@@ -70,7 +70,7 @@ typedef enum { LBF_I8 = 8, LBF_I16 = 16 } lbf_sample_bits;
 typedef enum { LBF_VOLTAGES = 0, LBF_STOKES_I = 1, LBF_STOKES_IQUV = 4 } lbf_output;
 
 /* Arithmetic of the beam former (the precision form of the beam former, Section 4.3 computed on
- * tensor cores): FP32 SIMT; FP16 tensor cores with three products (spectrum and weights both split
+ * tensor cores): FP32; FP16 tensor cores with three products (spectrum and weights both split
  * hi + lo: Whi Yhi + Wlo Yhi + Whi Ylo, FP32 accumulation, errors ~1e-6 relative); or FP16 tensor
  * cores with two products (spectrum split hi + lo, weights rounded to FP16 once: Whi Yhi + Whi Ylo,
  * two thirds of the MMA work; the weight rounding, <= 2^-12 per component, leaves Stokes I within
@@ -83,7 +83,10 @@ typedef enum { LBF_FP32 = 0, LBF_FP16_TC = 1, LBF_FP16_TC2 = 2 } lbf_precision;
  * or the register-tiled FP32 many-beam kernel with the beam tile -- 128 (MANY) or 64 (MANY64)
  * beams per CTA -- that leaves the fewest tile slots empty (a 64-beam slot weighed as 1.15 of a
  * 128-beam one).  With
- * LBF_FP16_TC or LBF_FP16_TC2, MANY and MANY64 both select the tensor-core kernel. */
+ * LBF_FP16_TC or LBF_FP16_TC2, MANY and MANY64 both select the tensor-core kernel.
+ * Of an FP32 plan FEW, MANY and MANY64 run the FP32 FMA kernel they name.  AUTO, up to 64 stations,
+ * runs all but few beams and some small blocks on the tensor cores instead, from FP16 slices of the
+ * FP32 operands (bf_split), no further from the 64-bit result than the FMA kernels. */
 typedef enum { LBF_BF_AUTO = 0, LBF_BF_FEW = 1, LBF_BF_MANY = 2, LBF_BF_MANY64 = 3 } lbf_bf_variant;
 
 /* The plan does not allocate the run_block scratch; the caller passes one to lbf_run_block_ws
@@ -125,9 +128,8 @@ typedef struct lbf_dims {
   int32_t d_max;              /* largest integer shift d_s, in samples */
   int32_t history_samples;    /* H = (L-1) N + d_max samples kept per (station, subband) */
   int32_t bf_kernel;          /* beam-former form of the plan: 1 few-beam, 2 many-beam FP32 (128-beam
-                                 tiles), 3 tensor core, 4 many-beam FP32 (64-beam tiles); up to 64
-                                 stations the FP32 forms of more than a few beams run on the tensor
-                                 cores from error-free FP16 slices, to FP32 accuracy */
+                                 tiles), 3 tensor core, 4 many-beam FP32 (64-beam tiles); the trace
+                                 names the kernel that ran (bf_split: see LBF_BF_AUTO) */
   size_t in_bytes;            /* bytes of one input block */
   size_t chan_bytes;          /* bytes of a chan buffer */
   size_t ct_bytes;            /* bytes of a ct buffer */
@@ -289,8 +291,8 @@ typedef struct lbf_trace {
   int32_t launches[16];        /* launches per kernel */
   double total_ms[16];         /* summed event time per kernel */
   char names[16][32];          /* kernel names: ppf, ppf_ct, hist_update, delay_ct, bf_few, bf_many,
-                                  stokes, ppf_ct16, bf_tc, ct_to_ct16, incoherent_ct16,
-                                  dedisperse, superstation */
+                                  bf_many64, bf_split, stokes, ppf_ct16, bf_tc, ct_to_ct16,
+                                  incoherent_ct16, dedisperse, superstation */
   int32_t dropped;             /* launches not recorded because max_launches was reached */
 } lbf_trace;
 lbf_status lbf_trace_begin(lbf_plan_t plan, int32_t max_launches);

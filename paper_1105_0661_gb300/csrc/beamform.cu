@@ -5,8 +5,9 @@
 // with w[b,s] = exp(+2 pi i f_c dtau[b,s]), f_c = f0_f + df_c.  The weights are generated per CTA
 // into shared memory from the plan's FP64-reduced phase tables (tables.cu) and an FP32 sincos.
 //
-// Up to 64 stations most of this runs as the split tensor-core kernel (bf_split.cu,
-// beamform_uses_split); the FP32 FMA kernels here serve few beams and more stations:
+// Under AUTO most of this runs up to 64 stations as the split tensor-core kernel (bf_split.cu,
+// beamform_uses_split); the FP32 FMA kernels here serve few beams, more stations and plans that name
+// one of them:
 //  * few-beam (bandwidth bound): one thread per spectrum m (both pols), weights broadcast from
 //    shared memory, one coalesced pass over the corner-turned input; Stokes integration over Q
 //    consecutive spectra is a warp-shuffle reduction across the lanes that hold them.
@@ -480,7 +481,8 @@ cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct,
   return cudaGetLastError();
 }
 
-// The split kernel takes the many-beam forms up to 64 stations, and of the few-beam form what would
+// A plan that names its variant gets that FMA kernel.  Under AUTO the split kernel takes the many-beam
+// forms up to 64 stations, and of the few-beam form what would
 // be two passes or more of the few-beam kernel over enough stations: its time hardly depends on the
 // beams up to 64, the few-beam kernel's grows with passes x stations.  Measured for 768 spectra,
 // few-beam / split: Stokes I, 16 subbands: 8 stations 16 beams 0.33 / 0.33 ms, 12 stations 16 beams
@@ -514,7 +516,7 @@ static int split_min_passes(const Geometry &g, int out_kind) {
 }
 
 bool beamform_uses_split(const Geometry &g, int variant, int out_kind) {
-  if (g.S > split_max_stations() || g.S < split_min_stations(g, out_kind)) return false;
+  if (!g.auto_bf || g.S > split_max_stations() || g.S < split_min_stations(g, out_kind)) return false;
   if (variant != 1) return true;
   if (g.inc && out_kind == OUT_STOKES_I && g.B <= 16) return false;
   return g.B > 8 && (g.B + 7) / 8 * g.S >= split_min_passes(g, out_kind);

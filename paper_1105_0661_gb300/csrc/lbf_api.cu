@@ -231,11 +231,11 @@ lbf_status check_call(lbf_plan_t p) {
 }
 
 enum KernelId { K_PPF = 0, K_PPF_CT, K_HIST, K_DELAY, K_BF_FEW, K_BF_MANY, K_STOKES, K_PPF_CT16, K_BF_TC,
-                K_CT16, K_INC16, K_DEDISP, K_SS, K_BF_MANY64, K_COUNT };
+                K_CT16, K_INC16, K_DEDISP, K_SS, K_BF_MANY64, K_BF_SPLIT, K_COUNT };
 static_assert(K_COUNT <= 16, "lbf_trace holds 16 kernels");
 const char *const kKernelNames[K_COUNT] = {"ppf", "ppf_ct", "hist_update", "delay_ct", "bf_few", "bf_many",
                                            "stokes", "ppf_ct16", "bf_tc", "ct_to_ct16", "incoherent_ct16",
-                                           "dedisperse", "superstation", "bf_many64"};
+                                           "dedisperse", "superstation", "bf_many64", "bf_split"};
 
 // Launch through `fn`, bracketed by trace events when a trace is active.
 template <typename Fn>
@@ -262,7 +262,11 @@ void trace_free(lbf_plan_t p) {
   p->tracing = false;
 }
 
-int bf_kernel_id(lbf_plan_t p) { return p->variant == 1 ? K_BF_FEW : p->variant == 3 ? K_BF_MANY64 : K_BF_MANY; }
+// the kernel launch_beamform runs
+int bf_kernel_id(lbf_plan_t p, int out_kind) {
+  if (lbf::beamform_uses_split(p->geometry(), p->variant, out_kind)) return K_BF_SPLIT;
+  return p->variant == 1 ? K_BF_FEW : p->variant == 3 ? K_BF_MANY64 : K_BF_MANY;
+}
 
 // The filter bank of one block with the next block's history, in one launch or two.
 cudaError_t filter_bank(lbf_plan_t p, int kernel, const lbf::Geometry &g, const void *d_in, float2 *chan, float2 *ct,
@@ -318,7 +322,7 @@ cudaError_t run_block_device(lbf_plan_t p, const void *d_in, void *d_out, void *
   if (e == cudaSuccess && out_free) e = cudaStreamWaitEvent(st, out_free, 0);
   if (e != cudaSuccess) return e;
   p->cur ^= 1;
-  return traced(p, bf_kernel_id(p), st,
+  return traced(p, bf_kernel_id(p, p->out_kind), st,
                 [&] { return lbf::launch_beamform(g, p->variant, p->out_kind, ct, d_out, st); });
 }
 
@@ -363,6 +367,7 @@ lbf_status lbf_plan(const lbf_config *cfg, lbf_plan_t *out) {
     p->variant = lbf::auto_bf_variant(p->B, p->S);
   else
     p->variant = cfg->bf_variant;
+  p->auto_bf = cfg->bf_variant == LBF_BF_AUTO;
   // Tensor cores only where the beam count makes the beam former a dense contraction: a
   // tensor-core plan with few beams (AUTO and B <= 8, or FEW asked for) runs the bandwidth-bound
   // few-beam kernel on the FP32 corner-turned block instead (Section 4.3: few beams stream the
@@ -565,7 +570,7 @@ lbf_status lbf_beamform(lbf_plan_t p, const void *d_ct, void *d_vol, void *strea
       return lbf::launch_bf_tc(g, lbf::OUT_VOLTAGES, &p->tmap[0], &p->tmap[1], static_cast<float *>(d_vol), p->d_err,
                                st, stall); }));
   }
-  return cuda_status(traced(p, bf_kernel_id(p), st, [&] {
+  return cuda_status(traced(p, bf_kernel_id(p, lbf::OUT_VOLTAGES), st, [&] {
     return lbf::launch_beamform(g, p->variant, lbf::OUT_VOLTAGES, (const float2 *)d_ct, d_vol, st); }));
 }
 
@@ -590,7 +595,7 @@ lbf_status lbf_beamform_stokes(lbf_plan_t p, const void *d_ct, float *d_out, voi
       p->stall_item = -1;
       return lbf::launch_bf_tc(g, p->out_kind, &p->tmap[0], &p->tmap[1], d_out, p->d_err, st, stall, inc); }));
   }
-  return cuda_status(traced(p, bf_kernel_id(p), st, [&] {
+  return cuda_status(traced(p, bf_kernel_id(p, p->out_kind), st, [&] {
     return lbf::launch_beamform(g, p->variant, p->out_kind, (const float2 *)d_ct, d_out, st); }));
 }
 

@@ -37,6 +37,7 @@ struct Geometry {
   const float *stepg = nullptr;
   int ct16_raw = 0;           // 1: the FP16 planes hold the filtered spectrum before the delay phase
                               // and bandpass, which the tensor-core weights then carry
+  int auto_bf = 0;                      // 1: bf_variant AUTO, launch_beamform chooses the kernel
   int *err = nullptr;                   // device error word: a bounded wait that gave up records here
   int pdl = 0;                          // 1: launch behind the previous kernel's tail (launch_behind)
   long long ppf_stall = -1;             // failure-detection test: this filter-bank CTA issues no input copies
@@ -200,7 +201,7 @@ struct SplitPlanRef {
 cudaError_t launch_bf_split(const SplitPlanRef *plans, int n, int out_kind, int Q, cudaStream_t st);
 int split_max_stations();
 int split_max_plans_per_launch();
-// whether launch_beamform runs `variant` of this observation as the split kernel
+// whether launch_beamform runs this observation (AUTO, `variant` of the FMA kernels) as the split kernel
 bool beamform_uses_split(const Geometry &g, int variant, int out_kind);
 // incoherent beam (index B of the Stokes output) from the FP32 corner-turned block
 cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct, float *out, cudaStream_t st);

@@ -33,7 +33,9 @@ def test_coherent_sums_are_exact_to_the_last_place(S):
     y[:, :, 0, :, 0] = 1
     p = Plan.from_workload(wl)
     o = torch.empty(p.shape("vol"), dtype=torch.complex64, device=dev)
+    p.trace_begin()
     p.beamform(torch.from_numpy(y).to(dev), o)
+    assert "bf_split" in p.trace_end()
     assert p.device_status() == 0
     p.close()
     v = o.cpu().numpy()                              # [B][F][N][P][M]

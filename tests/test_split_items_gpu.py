@@ -34,6 +34,7 @@ def test_quadrants_without_beams(S, B, M, Q, out):
     ob = O.observation_from_workload(wl)
     v = ob.beamform(ct.astype(np.complex128))
     dv = 8e-7 * S * np.abs(ct).max()
+    p.trace_begin()
     for _ in range(3):
         if out == "V":
             o = torch.full(p.shape("vol"), float("nan"), dtype=torch.complex64, device=dev)
@@ -46,4 +47,5 @@ def test_quadrants_without_beams(S, B, M, Q, out):
             # |dI| <= 2 |V| |dV| + |dV|^2 summed over pols and spectra
             assert np.all(np.abs(o.cpu().numpy() - ref) <= 4 * dv * (ref[:, :1] * Q) ** 0.5 + 4e-7 * ref[:, :1])
         assert p.device_status() == 0
+    assert [k for k in p.trace_end() if k.startswith("bf_")] == ["bf_split"]
     p.close()

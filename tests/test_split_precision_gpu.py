@@ -19,7 +19,7 @@ N = 256
 
 
 def _rms(S, M, gain, scale=1.0):
-    """RMS errors of the two kernels over 8 beams, relative to the RMS voltage; the kernels' traces."""
+    """RMS errors of the two kernels over 8 beams, relative to the RMS voltage."""
     from paper_1105_0661_gb300 import Plan, build_lib
     build_lib.build()
     dev = torch.device("cuda:0")
@@ -34,7 +34,9 @@ def _rms(S, M, gain, scale=1.0):
         wl = G.Workload("prec", xyz, G.subband_centres(1, 120e6), G.hex_beam_grid(40, 0.05)[:B], (0.3, 0.4), M * N, 1, "V")
         p = Plan.from_workload(wl)
         o = torch.empty(p.shape("vol"), dtype=torch.complex64, device=dev)
+        p.trace_begin()
         p.beamform(x, o)
+        assert ("bf_split" if B == 40 else "bf_few") in p.trace_end()
         assert p.device_status() == 0
         got = o.cpu().numpy()[:8].astype(np.complex128)
         if B == 40:
