@@ -464,9 +464,14 @@ lbf_status lbf_batch_tune(lbf_batch_t b, const void *const *d_in, void *const *d
   const int spcs[3] = {64, 256, 1024};
   // beam-former choices: 0 each plan's own; 1 plans with 9..64 beams switched between the few- and
   // many-beam kernels; 2 plans with more than 8 beams switched between the 128- and 64-beam tiles
-  std::vector<int> choice[3];
+  // (one that runs the same kernels as an earlier one is not timed: the split kernel serves a plan under
+  // either tile)
+  std::vector<int> choice[3], runs[3];
   bool has[3] = {true, false, false};
-  for (int k = 0; k < 3; ++k) choice[k].resize(n);
+  for (int k = 0; k < 3; ++k) {
+    choice[k].resize(n);
+    runs[k].resize(n);
+  }
   for (int i = 0; i < n; ++i) {
     lbf_plan_t p = b->plans[i];
     const int v = p->variant;
@@ -475,9 +480,13 @@ lbf_status lbf_batch_tune(lbf_batch_t b, const void *const *d_in, void *const *d
     const bool mid = fp32_many_ok && p->B <= 64;
     choice[1][i] = mid ? (v == 1 ? 2 : 1) : v;
     choice[2][i] = fp32_many_ok ? (v == 3 ? 2 : 3) : v;
-    has[1] = has[1] || mid;
-    has[2] = has[2] || fp32_many_ok;
+    for (int k = 0; k < 3; ++k) {
+      const int c = choice[k][i];
+      runs[k][i] = !p->tc && lbf::beamform_uses_split(p->geometry(), c, p->out_kind) ? 0 : c;
+    }
   }
+  has[1] = runs[1] != runs[0];
+  has[2] = runs[2] != runs[0] && runs[2] != runs[1];
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
