@@ -36,6 +36,11 @@
 // which spares the planes a second pass (127 beams of 30 subbands: 1.235 ms for
 // both, 1.227 + 0.928 apart).
 //
+// Quadrants without beams (the second M tile of a plan of up to 64 beams, say) are not drained: 17 beams of
+// 9 stations, 13 subbands, 87 windows of 4, whose staged rows cannot be stored 16 bytes wide and lost to
+// scattered stores otherwise: Stokes I 0.197 -> 0.187 ms, IQUV 0.317 -> 0.271 (scattered 0.191 and 0.270);
+// 40 beams 0.236 -> 0.205.
+//
 // The epilogue integrates each polarisation component over the window in registers (one shuffle
 // per spectrum for Stokes V) and combines the (Re, Im) row pair with two shuffles per window.
 // Every mbarrier wait is bounded: on expiry the kernel records an error code, stops issuing work,
@@ -670,11 +675,12 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
             load_weight_tables(pn, nfc / kN, nbb * kBeamsPerItem + mt * (kRows / 2) + quad * 16 + jq, ro, half, tab);
           if (!mbar_wait(accf_bar(mt), gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
           tc_fence_after();
-          const int b = bb * kBeamsPerItem + mt * (kRows / 2) + quad * 16 + jq;
+          const int b0 = bb * kBeamsPerItem + mt * (kRows / 2) + quad * 16;   // beam of lanes 0, 1
+          const int b = b0 + jq;
           const uint32_t taddr = tmem + lane_off + (uint32_t)(mt * kAccCols + h * 2 * kSpec + q2 * kSpecW);
           const int m0 = t * 2 * kSpec + h * kSpec + q2 * kSpecW;
-          if constexpr (NS == 0) {
-            const int b0 = bb * kBeamsPerItem + mt * (kRows / 2) + quad * 16;   // beam of lanes 0, 1
+          if (b0 >= p.B) {   // nothing to drain in a quadrant without beams
+          } else if constexpr (NS == 0) {
             const long long bstride = (long long)p.F * kN * kP * p.M;             // between beams
             float2 *const v0 = reinterpret_cast<float2 *>(p.out) + (((long long)b0 * p.F + f) * kN + c) * kP * p.M;
             drain_tile_v(taddr, m0, ro, jq, lane, p.M, p.B, b0, v0, bstride, p.vec != 0,
@@ -688,9 +694,9 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
           __syncwarp();
           if (lane == 0) mbar_arrive(acce_bar(mt));
           if constexpr (NS != 0 && !St::kOn) {   // the accumulator is free: write the short rows out
-            const int b0 = bb * kBeamsPerItem + mt * (kRows / 2) + quad * 16;
-            St::Rows::flush(stage_out + (warp - 2) * (St::Rows::kBytes / 4), lane, p.B - b0, m0 / Q, Mq,
-                            p.out + (((long long)b0 * NS * p.F + f) * kN + c) * Mq, NS * pstride, pstride);
+            if (b0 < p.B)
+              St::Rows::flush(stage_out + (warp - 2) * (St::Rows::kBytes / 4), lane, p.B - b0, m0 / Q, Mq,
+                              p.out + (((long long)b0 * NS * p.F + f) * kN + c) * Mq, NS * pstride, pstride);
           }
           if (boundary) {
             const uint32_t ta_hi = tmem + lane_off + wcol<kForm>(mt, (eit + 1) & 1);
