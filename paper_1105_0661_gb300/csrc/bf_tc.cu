@@ -607,7 +607,7 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
           const float bpc = p.bp ? __ldg(&p.bp[fc % kN]) : 1.f;
           float *const orow = p.out + ((long long)p.B * p.F * kN + fc) * (p.M / Q);
           for (int t = 0; t < p.ntiles; ++t) {
-            if (!mbar_wait(full_bar(s), ph, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+            if (!warp_wait(full_bar(s), ph, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
             if (mine)
               incoherent_atom<Q>(sbase + kBarBytes + (size_t)s * L.stage_max + (size_t)a * p.Kpad * 128,
                                  (uint32_t)p.stage_bytes / 2, p.S, lane, (2 * t + a) * kSpec, p.M, bpc * bpc, orow);
@@ -673,7 +673,7 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
           WeightTables<KS> tab;
           if (boundary)   // the next item's table values, in flight while the last accumulator fills
             load_weight_tables(pn, nfc / kN, nbb * kBeamsPerItem + mt * (kRows / 2) + quad * 16 + jq, ro, half, tab);
-          if (!mbar_wait(accf_bar(mt), gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+          if (!warp_wait(accf_bar(mt), gpar, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
           tc_fence_after();
           const int b0 = bb * kBeamsPerItem + mt * (kRows / 2) + quad * 16;   // beam of lanes 0, 1
           const int b = b0 + jq;
@@ -711,7 +711,7 @@ bf_tc_kernel(const __grid_constant__ TcLaunch L) {
           // both warps of the quadrant have staged their windows: write the rows out
           __syncwarp();
           if (lane == 0) mbar_arrive(pair_bar(quad));
-          if (!mbar_wait(pair_bar(quad), (uint32_t)fl & 1u, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
+          if (!warp_wait(pair_bar(quad), (uint32_t)fl & 1u, abort_flag)) { fail(abort_flag, p.err, ERR_EPILOGUE); ok = false; break; }
           flush_stage<NS, Q>(p, buf, frows, wbase);
           ++fl;
         }
