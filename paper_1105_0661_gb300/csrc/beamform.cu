@@ -481,45 +481,61 @@ cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct,
   return cudaGetLastError();
 }
 
-// A plan that names its variant gets that FMA kernel.  Under AUTO the split kernel takes the many-beam
-// forms up to 64 stations, and of the few-beam form what would
-// be two passes or more of the few-beam kernel over enough stations: its time hardly depends on the
-// beams up to 64, the few-beam kernel's grows with passes x stations.  Measured for 768 spectra,
-// few-beam / split: Stokes I, 16 subbands: 8 stations 16 beams 0.33 / 0.33 ms, 12 stations 16 beams
-// 0.40 / 0.35, 48 stations 16 beams 0.99 / 0.53 and 8 beams 0.51 / 0.51; voltages, 8 subbands: 12
-// stations 24 beams 0.29 / 0.30, 24 stations 12 beams 0.32 / 0.33, 48 stations 9 beams 0.58 / 0.37.
-// With a handful of stations the split kernel's weights (short blocks) and its epilogue (unintegrated
-// output, where the FMA kernels are bound by the output alone) weigh most; where the line lies, 4
-// subbands, 40 beams, many-beam kernel / split in us: Stokes I 768 spectra Q = 1, 4 stations 104 / 131,
-// 8 stations 162 / 132; 64 spectra, 12 stations 31 / 31; IQUV Q = 1, 768 spectra, 12 stations 268 / 300,
-// 16 stations 330 / 305, 128 spectra, 16 stations 51 / 54; voltages 768 spectra, 6 stations 144 / 154.
-// The incoherent beam costs the split kernel a pass of its own over the block, which the few-beam
-// kernel's one pass for up to 16 beams of Stokes I saves: 16 subbands, few-beam / split and the pass:
-// 12 beams of 16 stations 0.437 / 0.475 ms, of 64 1.20 / 1.26; 16 beams of 64 stations 1.25 / 1.28;
-// 24 beams of 16 stations 0.68 / 0.48.
-static int split_min_stations(const Geometry &g, int out_kind) {
-  const bool brief = g.M < 256;
-  if (out_kind == OUT_STOKES_IQUV && g.Q == 1) return brief ? 24 : 16;
-  if (out_kind == OUT_VOLTAGES || (out_kind == OUT_STOKES_I && g.Q <= 2)) return brief ? 16 : 8;
-  return g.M < 512 ? 8 : out_kind == OUT_STOKES_I && g.Q <= 4 ? 4 : 1;
+// Times of the three FP32 beam formers in us of one SM for one (subband, channel): least-squares fits of
+// their parts to 6200 measured launches (4 subbands; 1 to 64 stations, 63 to 768 spectra, 9 to 130
+// beams, every output and window), which they meet within 10 % (1st to 9th decile).  l: log2 of the
+// window.
+//  * few-beam kernel: a constant and the block's reads per pass of 8 beams (16 for 1.91 passes' worth),
+//    the detection per beam; m: spectra over the 256 of a CTA, padded to whole channels' threads.
+static float few_us(const Geometry &g, int out_kind, int l) {
+  const int step = kFewThreads >> few_log_channels(g.M, g.S, kFewBeams);
+  const float m = (float)((g.M + step - 1) / step * step) / kFewThreads;
+  const int p8 = (g.B + 7) / 8, p16 = (g.B + 15) / 16;
+  const float passes = out_kind == OUT_STOKES_I && 191 * p16 < 100 * p8 ? 1.91f * p16 : (float)p8;
+  const float detect = out_kind == OUT_STOKES_I ? 0.578f + 0.088f * l
+                     : out_kind == OUT_VOLTAGES ? 0.751f : l == 0 ? 2.237f : 3.865f + 0.372f * l;
+  return passes * (0.438f + 0.132f * g.S * m) + detect * g.B * m / 8;
 }
 
-// Passes of the few-beam kernel times stations from which the split kernel takes its beams: short
-// windows raise the split kernel's epilogue.  4 subbands of 768 spectra, few-beam / split as a ratio:
-// Stokes I Q = 4: 16 stations 2 passes 0.83, 12 stations 3 passes over 1; Q = 2: 32 stations 2 passes
-// 0.90, 24 stations 3 passes over 1; Q = 1: 24 stations 2 passes 0.97, 32 over 1; IQUV Q = 1: 24
-// stations 2 passes 0.85, 32 over 1, Q >= 2: over 1 from 24.
-static int split_min_passes(const Geometry &g, int out_kind) {
-  if (out_kind == OUT_VOLTAGES || g.Q == 1) return 56;
-  if (out_kind == OUT_STOKES_IQUV) return 24;
-  return g.Q == 2 ? 72 : g.Q <= 8 ? 36 : 24;
+//  * many-beam kernel: weights per beam tile (a 64-beam tile counted as 0.575 of a 128-beam one), FMAs
+//    and detection per pass of 32 spectra.
+static float many_us(const Geometry &g, int variant, int out_kind, int l) {
+  const float tiles = variant == 3 ? 0.575f * ((g.B + 63) / 64) : (float)((g.B + 127) / 128);
+  const float detect = out_kind == OUT_STOKES_I ? (l == 0 ? 0.404f : 0.861f)
+                     : out_kind == OUT_VOLTAGES ? 0.687f : l == 0 ? 1.056f : 2.564f + 0.292f * l;
+  return tiles * (1.277f + 0.073f * g.S + (g.M + 31) / 32 * (0.153f * g.S + detect));
 }
 
+//  * split kernel: weights per work item (a row of a block of 64 beams, or a part of it), conversion (more
+//    for rows read 8 bytes at a time) and epilogue per tile of 64 spectra; its persistent CTAs take the
+//    items in whole waves.  The incoherent beam is a pass of its own over the block there.
+static float split_us(const Geometry &g, int out_kind, int l) {
+  static const float kTileI[6] = {1.17f, 1.84f, 1.15f, 0.82f, 0.76f, 0.71f};
+  static const float kTileIquv[6] = {3.46f, 2.08f, 1.40f, 1.36f, 0.99f, 0.92f};
+  constexpr int kSms = 152;
+  const float tile = out_kind == OUT_VOLTAGES ? 1.53f : out_kind == OUT_STOKES_I ? kTileI[l] : kTileIquv[l];
+  const float k = (float)((2 * g.S + 15) / 16);
+  const int ntiles = (g.M + 63) / 64, blocks = (g.B + 63) / 64;
+  const long long rows = (long long)g.F * kN * blocks;
+  const int tpc = split_tiles_per_item(rows, ntiles, kSms), chunks = (ntiles + tpc - 1) / tpc;
+  const float waves = (float)((rows * chunks + kSms - 1) / kSms) * kSms / (float)(rows * chunks);
+  float us = waves * blocks * (chunks * (1.89f + 0.302f * k) + ntiles * (k * (g.M % 4 ? 0.292f : 0.197f) + tile));
+  if (g.inc && out_kind != OUT_VOLTAGES)
+    us += (float)((g.M + 255) / 256) * (0.09f * g.S + (out_kind == OUT_STOKES_IQUV ? 0.276f : 0.069f));
+  return us;
+}
+
+// A plan that names its variant gets that FMA kernel.  Under AUTO the split kernel takes more than 8
+// beams of up to 64 stations where it is the faster one by the fits above and by 5 % for their error.
+// Over the measured launches that costs 1 % against the faster kernel each time.  For example, 4
+// subbands, Stokes I over 16, 9 beams: 48 stations, 768 spectra: few-beam kernel 248 us, split 176; 12
+// stations, 64 spectra: 14 and 24.
 bool beamform_uses_split(const Geometry &g, int variant, int out_kind) {
-  if (!g.auto_bf || g.S > split_max_stations() || g.S < split_min_stations(g, out_kind)) return false;
-  if (variant != 1) return true;
-  if (g.inc && out_kind == OUT_STOKES_I && g.B <= 16) return false;
-  return g.B > 8 && (g.B + 7) / 8 * g.S >= split_min_passes(g, out_kind);
+  if (!g.auto_bf || g.S > split_max_stations() || g.B <= 8) return false;
+  int l = 0;
+  while ((1 << l) < g.Q) ++l;
+  const float fma = variant == 1 ? few_us(g, out_kind, l) : many_us(g, variant, out_kind, l);
+  return 1.05f * split_us(g, out_kind, l) < fma;
 }
 
 cudaError_t launch_beamform(const Geometry &g, int variant, int out_kind, const float2 *ct, void *out,

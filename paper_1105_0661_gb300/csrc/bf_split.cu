@@ -1015,11 +1015,8 @@ bool fill_plan(SpLaunch &L, int i, const Geometry &g, int out_kind, const float2
   p.stage_bytes = 6 * p.Kpad * 128;
   p.ntiles = (g.M + kTileSpec - 1) / kTileSpec;
   p.ipf = (g.B + kItemBeams - 1) / kItemBeams;
-  // whole (f, c) rows per item; an observation of few rows is cut along the spectra, in spans of
-  // whole output flushes (at most 4 tiles), so that every SM has a few items
   const long long rows = (long long)g.F * kN * p.ipf;
-  p.tpc = p.ntiles;
-  while (p.tpc > 4 && rows * ((p.ntiles + p.tpc - 1) / p.tpc) < 4ll * sms) p.tpc = ((p.tpc / 2 + 3) / 4) * 4;
+  p.tpc = split_tiles_per_item(rows, p.ntiles, sms);
   p.chunks = (p.ntiles + p.tpc - 1) / p.tpc;
   const long long items = rows * p.chunks;
   const long long first = i == 0 ? 0 : (long long)L.plan[i - 1].first_item + L.plan[i - 1].items;
@@ -1045,6 +1042,15 @@ bool fill_plan(SpLaunch &L, int i, const Geometry &g, int out_kind, const float2
 }  // namespace
 
 int split_max_stations() { return kMaxKpad / 2; }
+
+// Whole (f, c) rows per item; an observation of few rows is cut along the spectra, in spans of whole output
+// flushes (at most 4 tiles), so that every SM has a few items.
+int split_tiles_per_item(long long rows, int ntiles, int sms) {
+  int tpc = ntiles;
+  while (tpc > 4 && rows * ((ntiles + tpc - 1) / tpc) < 4ll * sms) tpc = ((tpc / 2 + 3) / 4) * 4;
+  return tpc;
+}
+
 int split_max_plans_per_launch() { return kMaxPlans; }
 
 cudaError_t launch_bf_split(const SplitPlanRef *plans, int n, int out_kind, int Q, cudaStream_t st) {

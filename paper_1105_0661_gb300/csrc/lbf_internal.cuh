@@ -200,6 +200,8 @@ struct SplitPlanRef {
 };
 cudaError_t launch_bf_split(const SplitPlanRef *plans, int n, int out_kind, int Q, cudaStream_t st);
 int split_max_stations();
+// tiles of 64 spectra per work item, for `rows` = (f, c, beam block) rows of `ntiles` on `sms` SMs
+int split_tiles_per_item(long long rows, int ntiles, int sms);
 int split_max_plans_per_launch();
 // whether launch_beamform runs this observation (AUTO, `variant` of the FMA kernels) as the split kernel
 bool beamform_uses_split(const Geometry &g, int variant, int out_kind);

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 N = 256
 
 
-@pytest.mark.parametrize("S,B,variant,candidates", [(24, 40, "auto", 4), (24, 130, "auto", 4), (8, 20, "auto", 7),
+@pytest.mark.parametrize("S,B,variant,candidates", [(24, 40, "auto", 4), (24, 130, "auto", 4), (16, 12, "auto", 7),
                                                     (24, 40, "many64", 10), (66, 40, "auto", 10), (66, 130, "auto", 7),
                                                     (24, 4, "auto", 4)])
 def test_candidates(S, B, variant, candidates):

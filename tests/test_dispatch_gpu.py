@@ -18,7 +18,8 @@ N = 256
     ("few", "fp32", 24, 20, 64, "I", "bf_few", "bf_few"), ("many", "fp32", 24, 40, 64, "I", "bf_many", "bf_many"),
     ("many64", "fp32", 24, 40, 64, "IQUV", "bf_many64", "bf_many64"), ("few", "fp32", 48, 130, 64, "IQUV", "bf_few", "bf_few"),
     ("auto", "fp32", 24, 40, 64, "I", "bf_split", "bf_split"), ("auto", "fp32", 24, 8, 64, "I", "bf_few", "bf_few"),
-    ("auto", "fp32", 9, 40, 64, "I", "bf_split", "bf_many64"), ("auto", "fp32", 65, 40, 64, "I", "bf_many64", "bf_many64"),
+    ("auto", "fp32", 32, 9, 64, "I", "bf_few", "bf_few"),
+    ("auto", "fp32", 19, 40, 64, "I", "bf_split", "bf_many64"), ("auto", "fp32", 65, 40, 64, "I", "bf_many64", "bf_many64"),
     ("auto", "fp32", 65, 127, 64, "I", "bf_many", "bf_many"), ("few", "fp16tc", 24, 40, 64, "I", "bf_few", "bf_few")])
 def test_kernel_that_runs(variant, prec, S, B, M, out, stokes, volts):
     from paper_1105_0661_gb300 import Plan, build_lib

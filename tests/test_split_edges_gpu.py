@@ -19,15 +19,15 @@ pytestmark = pytest.mark.gpu
 N = 256
 
 
-def _wl(S, B, M, Q, out):
+def _wl(S, B, M, Q, out, F=1):
     rng = np.random.default_rng(S)
-    return G.Workload("edges", G.lofar_positions(rng, S // 2, S - S // 2), G.subband_centres(1, 120e6),
+    return G.Workload("edges", G.lofar_positions(rng, S // 2, S - S // 2), G.subband_centres(F, 120e6),
                       G.hex_beam_grid(B, 0.05), (0.3, 0.4), M * N, Q, out)
 
 
-def _ct(S, M, seed):
+def _ct(S, M, seed, F=1):
     rng = np.random.default_rng(seed)
-    shape = (1, N, S, 2, M)
+    shape = (F, N, S, 2, M)
     return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
 
 
@@ -46,25 +46,26 @@ def _run(wl, ct, kernel="bf_split", **over):
     return o.cpu().numpy()
 
 
-@pytest.mark.parametrize("S,B,M", [(8, 33, 257), (8, 64, 256), (9, 65, 510), (16, 40, 258), (17, 127, 63), (24, 65, 1),
-                                   (24, 129, 65), (31, 40, 130), (33, 40, 64), (40, 33, 20), (48, 133, 255), (49, 40, 66),
-                                   (57, 40, 65), (64, 50, 320), (64, 64, 7)])
-def test_voltages(S, B, M):
-    ct = _ct(S, M, 1)
-    wl = _wl(S, B, M, 1, "V")
+@pytest.mark.parametrize("S,B,M,F", [(9, 60, 512, 4), (16, 40, 258, 2), (20, 40, 129, 4), (24, 129, 65, 2), (31, 40, 130, 1),
+                                     (33, 40, 64, 1), (40, 33, 36, 1), (48, 133, 255, 1), (49, 40, 66, 1), (57, 40, 65, 1),
+                                     (64, 50, 320, 1), (64, 64, 33, 1), (64, 64, 7, 4)])
+def test_voltages(S, B, M, F):
+    ct = _ct(S, M, 1, F)
+    wl = _wl(S, B, M, 1, "V", F)
     ref = O.observation_from_workload(wl).beamform(ct.astype(np.complex128))
     peak = np.abs(ct).max(axis=2)[None].astype(np.float64)
     assert np.all(np.abs(_run(wl, ct) - ref) <= 2e-7 * S * peak + 2.0 ** -23 * np.abs(ref))
 
 
-@pytest.mark.parametrize("S,B,M,Q,out", [(1, 40, 512, 8, "I"), (2, 65, 544, 16, "I"), (1, 40, 512, 2, "IQUV"), (3, 40, 514, 2, "IQUV"),
-                                         (4, 70, 516, 4, "I"), (5, 40, 512, 32, "IQUV"), (7, 40, 520, 8, "IQUV"), (8, 40, 256, 2, "I"),
-                                         (8, 33, 257, 1, "I"), (16, 40, 255, 1, "I"), (16, 40, 257, 1, "IQUV"), (24, 40, 41, 1, "IQUV"),
-                                         (24, 129, 66, 2, "I"), (50, 40, 66, 2, "IQUV"), (56, 40, 68, 4, "IQUV"), (64, 40, 72, 8, "IQUV"),
-                                         (64, 70, 160, 32, "I"), (64, 40, 63, 1, "IQUV")])
-def test_stokes(S, B, M, Q, out):
-    ct = _ct(S, M, 2)
-    wl = _wl(S, B, M, Q, out)
+@pytest.mark.parametrize("S,B,M,Q,out,F", [
+    (1, 40, 768, 32, "I", 4), (2, 64, 544, 16, "I", 4), (1, 40, 512, 2, "IQUV", 1), (3, 40, 514, 2, "IQUV", 2),
+    (4, 32, 516, 4, "I", 4), (5, 40, 512, 32, "IQUV", 1), (5, 65, 512, 32, "I", 1), (7, 40, 520, 8, "IQUV", 1),
+    (8, 32, 257, 1, "I", 2), (16, 40, 255, 1, "I", 1), (16, 24, 257, 1, "IQUV", 4), (48, 40, 66, 1, "IQUV", 4),
+    (24, 129, 66, 2, "I", 2), (50, 40, 66, 2, "IQUV", 1), (56, 40, 68, 4, "IQUV", 1), (64, 40, 72, 8, "IQUV", 1),
+    (64, 70, 160, 32, "I", 1), (64, 40, 63, 1, "IQUV", 1)])
+def test_stokes(S, B, M, Q, out, F):
+    ct = _ct(S, M, 2, F)
+    wl = _wl(S, B, M, Q, out, F)
     ob = O.observation_from_workload(wl)
     ref = ob.stokes(ob.beamform(ct.astype(np.complex128)))
     dv = 2e-7 * S * np.abs(ct).max()
@@ -90,8 +91,8 @@ def test_infinities_and_nans_stay_in_their_columns(out, Q, M):
 
 @pytest.mark.parametrize("out,Q", [("I", 1), ("I", 8), ("IQUV", 4)])
 def test_incoherent_beam_beside_it(out, Q):
-    ct = _ct(24, 96, 5)
-    wl = _wl(24, 40, 96, Q, out)
+    ct = _ct(24, 128, 5)
+    wl = _wl(24, 40, 128, Q, out)
     got = _run(wl, ct, incoherent_beam=True)
     inc = O.observation_from_workload(wl, incoherent_beam=True).incoherent(ct.astype(np.complex128))
     assert np.all(np.abs(got[-1] - inc) <= 1e-5 * inc[:1])

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 N = 256
 
 
-def _plan(S, B, variant, prec, M=32):
+def _plan(S, B, variant, prec, M=64):
     from paper_1105_0661_gb300 import Plan
     rng = np.random.default_rng(S)
     wl = G.Workload("thr", G.lofar_positions(rng, S // 2, S - S // 2), G.subband_centres(1, 120e6),
