@@ -368,6 +368,7 @@ lbf_status lbf_plan(const lbf_config *cfg, lbf_plan_t *out) {
   else
     p->variant = cfg->bf_variant;
   p->auto_bf = cfg->bf_variant == LBF_BF_AUTO;
+  p->ppf_spc = lbf::ppf_spectra_per_cta(p->S, p->F, p->M);
   // Tensor cores only where the beam count makes the beam former a dense contraction: a
   // tensor-core plan with few beams (AUTO and B <= 8, or FEW asked for) runs the bandwidth-bound
   // few-beam kernel on the FP32 corner-turned block instead (Section 4.3: few beams stream the

@@ -37,6 +37,7 @@ struct Geometry {
   const float *stepg = nullptr;
   int ct16_raw = 0;           // 1: the FP16 planes hold the filtered spectrum before the delay phase
                               // and bandpass, which the tensor-core weights then carry
+  int ppf_spc = 0;                      // spectra per filter-bank CTA (ppf_spectra_per_cta)
   int auto_bf = 0;                      // 1: bf_variant AUTO, launch_beamform chooses the kernel
   int *err = nullptr;                   // device error word: a bounded wait that gave up records here
   int pdl = 0;                          // 1: launch behind the previous kernel's tail (launch_behind)
@@ -105,6 +106,8 @@ struct BfGroup {
 // a1-a3 (+ a4 when ct or ct16 is given): filter bank; reads history `hist`, block `in`.
 // and, where ppf_fuses_history(g) and new_hist is given, writes the next block's history to it
 bool ppf_fuses_history(const Geometry &g);
+// spectra per CTA of a plan's own filter bank
+int ppf_spectra_per_cta(int S, int F, int M);
 cudaError_t launch_ppf(const Geometry &g, int bits, const void *in, const void *hist, void *new_hist,
                        float2 *chan, float2 *ct, cudaStream_t st, const Ct16Out *ct16 = nullptr);
 // batch: persistent grouped filter bank (FP32 corner-turned output), history update, beam former.

@@ -17,6 +17,7 @@ struct lbf_plan_s {
   int device = 0;
   int S = 0, F = 0, N = 0, L = 0, B = 0, T = 0, M = 0, Q = 1, nS = 0, bits = 16;
   int out_kind = 0, variant = 1, d_max = 0, H = 0;
+  int ppf_spc = 0;              // spectra per filter-bank CTA
   bool auto_bf = false;         // bf_variant AUTO: the split kernel may take the FP32 beam former
   double fs = 0.0;
   std::vector<int32_t> n_shift, d_shift;
@@ -73,6 +74,7 @@ struct lbf_plan_s {
     g.tc_wlo = tc_wlo;
     g.err = d_err;
     g.auto_bf = auto_bf;
+    g.ppf_spc = ppf_spc;
     return g;
   }
 };

@@ -785,14 +785,19 @@ __global__ void __launch_bounds__(256) hist_group_kernel(const PpfGroup *__restr
 // the whole stream for the LOFAR block, one tile for a few streams.  With at least 16 waves' worth of CTAs
 // wherever M allowed them, whatever the last wave held, 240 streams of 8 tiles took 0.109 ms against 0.074
 // here, 384 of 48 tiles 0.516 against 0.482, 1073 of 16 tiles 0.501 against 0.488; 2928 of 48 the same.
-int spectra_per_cta(const Geometry &g) {
+// Tried once per plan, from one span length to the next shorter one: every number of spans at every launch
+// held up the host for 10 us (one stream of 2432 tiles).
+}  // namespace
+
+int ppf_spectra_per_cta(int S, int F, int M) {
   constexpr long long kSms = 152;
-  const long long streams = (long long)g.S * g.F;
-  const int ntiles = (g.M + kTile - 1) / kTile;
+  const long long streams = (long long)S * F;
+  const int ntiles = (M + kTile - 1) / kTile;
   long long best = 0;
   int best_tpc = ntiles;
-  for (int ch = 1; ch <= ntiles && (ch == 1 || streams * (ch - 1) < kSms * 16); ++ch) {
-    const int tpc = (ntiles + ch - 1) / ch;
+  for (int ch = 1, tpc = ntiles; ch <= ntiles && (ch == 1 || streams * (ch - 1) < kSms * 16);
+       ch = tpc > 1 ? (ntiles + tpc - 2) / (tpc - 1) : ntiles + 1) {
+    tpc = (ntiles + ch - 1) / ch;
     const long long ctas = streams * ((ntiles + tpc - 1) / tpc);
     const long long cost = (ctas + kSms - 1) / kSms * (2 * tpc + 3);
     if (best == 0 || cost < best) {
@@ -803,13 +808,15 @@ int spectra_per_cta(const Geometry &g) {
   return (best_tpc > 0 ? best_tpc : 1) * kTile;
 }
 
+namespace {
+
 template <int BITS, int MODE, bool kTma>
 cudaError_t launch_ppf_t(const Geometry &g, const void *in, const void *hist, void *nhist, PpfOut po, const PpfMaps &maps,
                          cudaStream_t st) {
   using word = typename SampleIO<BITS>::word;
   const long long streams = (long long)g.S * g.F;   // one CTA: both polarisations
   if (streams == 0 || g.M == 0) return cudaSuccess;
-  const int spc = spectra_per_cta(g);
+  const int spc = g.ppf_spc;
   const int chunks = (g.M + spc - 1) / spc;
   const long long ctas = streams * chunks;
   if (ctas == 0) return cudaSuccess;

@@ -183,6 +183,7 @@ extern "C" lbf_status lbf_run_block_static(const lbf_config *c, const void *d_in
   g.phase0 = reinterpret_cast<const int *>(tab + tm.phase0);
   g.step = reinterpret_cast<const float *>(tab + tm.step);
   g.err = reinterpret_cast<int *>(tab + tm.err);
+  g.ppf_spc = lbf::ppf_spectra_per_cta(S, F, M);
   g.auto_bf = c->bf_variant == LBF_BF_AUTO;
   const int out_kind = c->output == LBF_STOKES_I ? lbf::OUT_STOKES_I
                      : c->output == LBF_STOKES_IQUV ? lbf::OUT_STOKES_IQUV : lbf::OUT_VOLTAGES;
