@@ -57,6 +57,8 @@
 // waits (bounded) for its MMAs in flight, frees TMEM and returns.  The MMA thread, the evaluators and
 // the converters wait suspended; the epilogue polls (suspended waits cost it up to 70 % on short
 // items).
+#include <atomic>
+
 #include "tc_ptx.cuh"
 
 namespace lbf {
@@ -968,12 +970,16 @@ cudaError_t launch_q(SpLaunch &L, int grid, cudaStream_t st) {
   int smem = kFixed + L.nstages * L.stage_max + Stage<NS, Q>::kBytes + wstage;
   if (smem < kMinSmem) smem = kMinSmem;
   // the register split of the kernel's warpgroups draws on what the CTA was launched with
-  static const int regs = [&] {
+  static std::atomic<int> regs{0};   // of this kernel, once known
+  cudaError_t e = cudaSuccess;
+  if (regs.load(std::memory_order_relaxed) == 0) {
     cudaFuncAttributes a;
-    return cudaFuncGetAttributes(&a, kern) == cudaSuccess ? a.numRegs : 0;
-  }();
-  if (regs < kLaunchRegs) return cudaErrorInvalidConfiguration;
-  cudaError_t e = allow_shared(kern, smem);
+    e = cudaFuncGetAttributes(&a, kern);
+    if (e != cudaSuccess) return e;
+    regs.store(a.numRegs, std::memory_order_relaxed);
+  }
+  if (regs.load(std::memory_order_relaxed) < kLaunchRegs) return cudaErrorInvalidConfiguration;
+  e = allow_shared(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<grid, kThreads, smem, st>>>(L);
   return cudaGetLastError();
@@ -1001,11 +1007,9 @@ cudaError_t launch_kind(SpLaunch &L, int out_kind, int Q, int grid, cudaStream_t
 }
 
 int sm_count() {
-  static int n[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!n[dev] && cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n[dev] = 0;
-  return n[dev];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? n : 0;
 }
 
 bool fill_plan(SpLaunch &L, int i, const Geometry &g, int out_kind, const float2 *ct, void *out, int sms) {

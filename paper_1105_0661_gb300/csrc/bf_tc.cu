@@ -759,11 +759,9 @@ cudaError_t launch_ns(int Q, TcLaunch &L, int grid, cudaStream_t st) {
 }
 
 int sm_count() {
-  static int n[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!n[dev] && cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n[dev] = 0;
-  return n[dev];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? n : 0;
 }
 
 // Plan i of a launch: its parameters from the geometry, its work items after the previous plans'.
