@@ -46,10 +46,11 @@
 //  * epilogue warps (8): warp w serves TMEM lane quadrant w % 4 and one 32-spectrum half.  They take
 //    D2 into registers while the MMAs fill D1, and D1 while the MMAs fill the next tile's D2, so
 //    that one accumulator of each suffices (256 TMEM columns, next to 3 x 64 of weight slices).
-// What bounds it: the latency of the converters' chain and the issue slots; the MMAs (64 cycles each)
-// take 2300 of a tile's 4000 cycles at 48 stations.  127 beams of the LOFAR block: 86.2 ms in FP32
-// FMAs, 20.5 here; 37 beams of 30 subbands: 5.5 ms and 1.29; voltages of 127 beams, 16 subbands: 5.7 ms
-// and 1.87.  The ring holds two stages up to 56 stations and one beyond (64 stations, 127 beams, 8
+// What bounds it: the issue slots (ncu, 8 subbands of the LOFAR block: 56 % of them used, 9000 warp
+// instructions per tile of 64 beams, most of them the converters') and the latency of the converters'
+// chain; the MMAs (64 cycles each) take 57 % of a tile's 4000 cycles.  127 beams of the LOFAR block: 86.2
+// ms in FP32 FMAs, 20.5 here; 37 beams of 30 subbands: 5.5 ms and 1.29; voltages of 127 beams, 16 subbands:
+// 5.7 ms and 1.87.  The ring holds two stages up to 56 stations and one beyond (64 stations, 127 beams, 8
 // subbands: 1.20 ms against 0.74 for 56).  Measured and dropped: stages of two slices that share a third
 // one (64 stations 1.20 -> 1.10 ms, 48 stations 0.67 -> 0.71: registers), stages released by halves (an
 // MMA of 64 columns takes as long as one of 128: 48 stations 0.67 -> 1.08).
@@ -71,7 +72,9 @@ constexpr int kTileSpec = 2 * kSpec;        // 64 spectra per tile
 constexpr int kEpiWarps = 8, kConvWarps = 8;
 constexpr int kGroup = kConvWarps / 2;      // converter warps per half tile
 constexpr int kThreads = 128 + 32 * (kEpiWarps + kConvWarps);   // warpgroup 0: MMA issuer and 3 weight evaluators
-constexpr int kMaxStages = 4;
+// a third and fourth stage gain nothing and take the L1 cache from the voltage rows (24 stations, 61 beams,
+// 16 subbands: 0.90 ms with four, 0.78 with two)
+constexpr int kMaxStages = 2;
 constexpr int kBarBytes = 1024;
 constexpr int kSlots = 8;                   // column-scale ring: more than the stages + 3 tiles in flight
 constexpr int kScaleBytes = kSlots * kCols * 4;
@@ -91,9 +94,10 @@ constexpr float kWUnit = 128.f;
 constexpr float kMagic = 12582912.f;        // 1.5 * 2^23: x + kMagic rounds x to an integer
 constexpr float kMagic2 = 6144.f;           // 1.5 * 2^12: x + kMagic2 rounds x to a multiple of 2^-11
 constexpr int kPrefetch = 4;                // tiles an L2 prefetch runs ahead of the loads
-// registers per thread after the split of what the CTA is launched with (640 x 96 = 61440):
-// 128 x 40 + 256 x 112 + 256 x 104 = 60416.  The compiler allocates each section by its own share: with
-// 96 for the converters of three slices all kernels spilled 300 bytes and more a thread, with 104 up to 40
+// Registers per thread after the split of what the CTA is launched with (640 x 96 = 61440): 128 x 40 +
+// 256 x 112 (epilogue) + 256 x 104 (converters) = 60416.  The compiler allocates each section by its own
+// share: with 120 and 96 all kernels spilled 300 bytes and more a thread, so up to 90.  (The voltage
+// epilogue of 24 stations gains 3 % from 120, but 64 stations lose 40 % with 96 for the converters.)
 constexpr int kLaunchRegs = 96;
 
 struct SpParams {
