@@ -483,8 +483,8 @@ cudaError_t launch_incoherent(const Geometry &g, int out_kind, const float2 *ct,
 
 // Times of the three FP32 beam formers in us of one SM for one (subband, channel): least-squares fits of
 // their parts to 6200 measured launches (4 subbands; 1 to 64 stations, 63 to 768 spectra, 9 to 130
-// beams, every output and window), which they meet within 10 % (1st to 9th decile).  l: log2 of the
-// window.
+// beams, every output and window): from the 1st to the 9th decile the split and the many-beam kernel lie
+// within 10 % of them, the few-beam kernel within 21 %.  l: log2 of the window.
 //  * few-beam kernel: a constant and the block's reads per pass of 8 beams (16 for 1.91 passes' worth),
 //    the detection per beam; m: spectra over the 256 of a CTA, padded to whole channels' threads.
 static float few_us(const Geometry &g, int out_kind, int l) {
@@ -527,11 +527,11 @@ static float split_us(const Geometry &g, int out_kind, int l) {
 
 // A plan that names its variant gets that FMA kernel.  Under AUTO the split kernel takes more than 8
 // beams of up to 64 stations where it is the faster one by the fits above and by 5 % for their error.
-// Over the measured launches that costs 1 % against the faster kernel each time.  For example, 4
-// subbands, Stokes I over 16, 9 beams: 48 stations, 768 spectra: few-beam kernel 248 us, split 176; 12
-// stations, 64 spectra: 14 and 24.
+// Over launches of 1, 4 and 16 subbands that costs 1 to 2 % against the faster kernel each time.  For
+// example, 4 subbands, Stokes I over 16, 9 beams: 48 stations, 768 spectra: few-beam kernel 248 us, split
+// 176; 12 stations, 64 spectra: 14 and 24.
 bool beamform_uses_split(const Geometry &g, int variant, int out_kind) {
-  if (!g.auto_bf || g.S > split_max_stations() || g.B <= 8) return false;
+  if (!g.auto_bf || g.S > split_max_stations() || g.B <= 8 || g.M == 0) return false;
   int l = 0;
   while ((1 << l) < g.Q) ++l;
   const float fma = variant == 1 ? few_us(g, out_kind, l) : many_us(g, variant, out_kind, l);

@@ -41,3 +41,25 @@ def test_kernel_that_runs(variant, prec, S, B, M, out, stokes, volts):
     assert stokes in p.trace_end()
     assert p.device_status() == 0
     p.close()
+
+
+def test_empty_block_beside_others_in_a_batch():
+    """A plan of no spectra takes no kernel (its cost is not asked for), alone or in a batch."""
+    from paper_1105_0661_gb300 import Batch, Plan, build_lib
+    build_lib.build()
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(1)
+    plans = [Plan.from_workload(G.Workload("empty", G.lofar_positions(rng, 12, 12), G.subband_centres(1, 120e6),
+                                           G.hex_beam_grid(40, 0.05), (0.3, 0.4), M * N, 1, "I")) for M in (0, 64)]
+    x = [torch.zeros(max(1, p.dims.in_bytes // 2), dtype=torch.int16, device=dev) for p in plans]
+    o = [torch.ones(max(1, p.dims.out_bytes // 4), dtype=torch.float32, device=dev) for p in plans]
+    b = Batch(plans)
+    b.run(x, o)
+    torch.cuda.synchronize()
+    assert o[0].item() == 1.0 and torch.count_nonzero(o[1]).item() == 0
+    plans[0].trace_begin()
+    plans[0].run_block(x[0], o[0])
+    assert [k for k in plans[0].trace_end() if not k.startswith("_")] == []
+    b.close()
+    for p in plans:
+        p.close()
