@@ -5,7 +5,7 @@
 //
 // Why: the beam former of B beams does 16 B flop per station-sample.  In FP32 FMAs that is bound by
 // the FMA pipe from about 10 beams on (80 TFLOP/s: 58 ms for the 127-beam LOFAR block), while the
-// block could be read in 5.4 ms and its six FP16 products take 12 ms at the tensor-core rate.
+// block could be read in 5.4 ms and its six FP16 products take 15 ms at the measured tensor-core rate.
 //
 // The slices.  The tensor cores add FP16 products exactly but truncate the FP32 accumulator toward
 // zero as they go; that bias does not average out over an integration window, and is why the
@@ -19,7 +19,7 @@
 //  * D1 = W1 Y1 never rounds: |w1| < 2^7.01 and |y1| <= 2^10.5 keep a station's term below 2^17.51 and
 //    the sum of 64 stations in phase below 2^23.51; D2 = W2 Y1 + W3 Y1 + W1 Y2 + W2 Y2 + W1 Y3
 //    accumulates apart from it, 2^7 smaller and more, so that its truncation is below the result's
-//    last bit; the products left out are below 2^-30 of the peak;
+//    last bit; the products left out are below 2^-28 of the peak;
 //  * V = (D1 + D2) 2^-e in FP32.
 // What remains is the rounding of V and of the FP32 weights, where the FMA kernels round the
 // accumulator at every station.  RMS error of the voltages against 64 bits for a given block, FMA
